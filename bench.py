@@ -378,6 +378,7 @@ def measure_frames(cfg: int, args, dev: str, local: int, ws: int, l2_peak: float
         step()
     ctx.synchronize()
     hyp_step, samples_step = ctx.counters()
+    sweep_samples, prop_samples = ctx.samples_taken()    # what the kernels gathered to decide them
     ctx.profile_read()                                   # reset stage timers / launch counts
     ctx.profile_enable(True)
 
@@ -408,13 +409,11 @@ def measure_frames(cfg: int, args, dev: str, local: int, ws: int, l2_peak: float
     ctx.synchronize()
     ms_local = float(np.mean(step_ms))
     ms, value = replica_reduce(ms_local, hyp_step, ws, dev)
-    _, samples_per_s = replica_reduce(ms_local, samples_step, ws, dev)
+    _, samples_per_s = replica_reduce(ms_local, sweep_samples + prop_samples, ws, dev)
 
     # dominant kernel and its roofline
     stage_ms = {k: v[0] / args.steps for k, v in prof.items()}
     stage_launches = {k: v[1] / args.steps for k, v in prof.items()}
-    sweep_samples = int(params["num_labels"]) * V * H * W * min(V - 1, 8)
-    prop_samples = samples_step - sweep_samples
     dom = max(("sweep", "propagate"), key=lambda k: stage_ms[k])
     dom_samples = sweep_samples if dom == "sweep" else prop_samples
     launches = max(stage_launches[dom], 1)
@@ -423,6 +422,7 @@ def measure_frames(cfg: int, args, dev: str, local: int, ws: int, l2_peak: float
                            f"config{cfg}@{args.scale:g}", l2_peak)
     res = {"workload": workload_name(cfg, lf), "value": value, "ms_per_step": ms, "ms_per_view": ms / V,
            "samples_per_s": samples_per_s, "hypotheses_per_step": hyp_step, "samples_per_step": samples_step,
+           "samples_taken_per_step": sweep_samples + prop_samples,
            "stage_ms": stage_ms, "wall_s": wall, "gpu_launches": int(sum(v[1] for v in prof.values())),
            "roofline": roofline, "clocks": clock_info}
 
@@ -587,6 +587,7 @@ def run_ours_batch(args):
         out = ctx.estimate_batch(items, out=out, options=TUNE)
     ctx.synchronize()
     hyp_step, samples_step = ctx.counters()
+    sweep_samples, prop_samples = ctx.samples_taken()
     ctx.profile_read()
     ctx.profile_enable(True)
 
@@ -613,12 +614,9 @@ def run_ours_batch(args):
     prof = ctx.profile_read()
     ctx.profile_enable(False)
     ms, value = replica_reduce(ms_local, hyp_step, ws, dev)
-    _, samples_per_s = replica_reduce(ms_local, samples_step, ws, dev)
+    _, samples_per_s = replica_reduce(ms_local, sweep_samples + prop_samples, ws, dev)
     stage_ms = {k: v[0] / args.steps for k, v in prof.items()}
     stage_launches = {k: v[1] / args.steps for k, v in prof.items()}
-    sweep_samples = sum(int(m.params["num_labels"]) * m.rig.V * m.rig.W * m.rig.H * min(m.rig.V - 1, 8)
-                        for m in mix)
-    prop_samples = samples_step - sweep_samples
     dom = max(("sweep", "propagate"), key=lambda k: stage_ms[k])
     dom_samples = sweep_samples if dom == "sweep" else prop_samples
     launches = max(stage_launches[dom], 1)
@@ -632,7 +630,8 @@ def run_ours_batch(args):
                        "l2": "flushed between steps (256 MiB write)",
                        "inputs": "device-resident", "parallelism": f"replicas x{ws}"},
             "samples_per_s": samples_per_s, "hypotheses_per_step": hyp_step,
-            "samples_per_step": samples_step, "stage_ms": stage_ms,
+            "samples_per_step": samples_step,
+           "samples_taken_per_step": sweep_samples + prop_samples, "stage_ms": stage_ms,
             "gpu_launches": int(sum(v[1] for v in prof.values())), "launch_config": ctx.launch_config(),
             "roofline": roofline, "clocks": clock_info, "input_generation_s": t_gen}
     # the same light fields through lfd_estimate one after another (the plain

@@ -481,9 +481,14 @@ lfd_status lfd_server_import_state(lfd_server *srv, int32_t rig_id, const float 
  * (LFD_ERR_DEVICE_CHECK) raised by this context's kernels; clears them. */
 lfd_status lfd_synchronize(lfd_ctx *ctx, void *stream);
 
-/* Hypotheses scored and pixel-view samples taken by this context's kernels
- * since the last lfd_set_input / lfd_estimate (synchronous). */
+/* Hypotheses scored by this context's kernels since the last lfd_set_input /
+ * lfd_estimate, and the pixel-view samples their sums comprise (synchronous).
+ * A hypothesis that is decided before its sum is complete, because no
+ * completion could make it the best, counts in full. */
 lfd_status lfd_counters(lfd_ctx *ctx, uint64_t *hypotheses, uint64_t *samples, void *stream);
+/* Pixel-view samples the sweep and the refinement took to decide them (at
+ * most the samples of lfd_counters; synchronous). */
+lfd_status lfd_samples_taken(lfd_ctx *ctx, uint64_t *sweep, uint64_t *refine, void *stream);
 
 /* ---- tracing ------------------------------------------------------------ */
 

@@ -318,6 +318,7 @@ __device__ __forceinline__ void sweep_sp(const Workspace &w, const Consts &c, in
         if (label_out) label_out[gs] = bk;
         atomicAdd(&w.ctr->hyp, (unsigned long long)L);
         atomicAdd(&w.ctr->samples, (unsigned long long)L * n * nnb);
+        atomicAdd(&w.ctr->taken_sweep, (unsigned long long)L * n * nnb);
     }
 }
 

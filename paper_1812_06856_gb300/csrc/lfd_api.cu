@@ -3,6 +3,7 @@
 #include <algorithm>
 #include <cmath>
 #include <cstdarg>
+#include <cstddef>
 #include <cstdio>
 #include <cstring>
 #include <new>
@@ -1481,7 +1482,7 @@ lfd_status estimate_batch_impl(lfd_ctx *ctx, int32_t n, const lfd_lightfield *lf
         // the launch shapes are timed on this input, bound outside any capture
         if ((s = enqueue_input(ctx, st, true)) != LFD_OK) return s;
         if ((s = autotune(ctx, st)) != LFD_OK) return s;
-        LFD_CUDA(cudaMemsetAsync(ctx->d_ctr, 0, 2 * sizeof(unsigned long long), st));
+        LFD_CUDA(cudaMemsetAsync(ctx->d_ctr, 0, offsetof(DevCounters, status), st));
         ctx->tuned_sig = sig;
     }
 
@@ -1818,6 +1819,19 @@ lfd_status lfd_counters(lfd_ctx *ctx, uint64_t *hypotheses, uint64_t *samples, v
     LFD_CUDA(cudaMemcpy(&h, ctx->d_ctr, sizeof(h), cudaMemcpyDeviceToHost));
     if (hypotheses) *hypotheses = h.hyp;
     if (samples) *samples = h.samples;
+    return LFD_OK;
+}
+
+lfd_status lfd_samples_taken(lfd_ctx *ctx, uint64_t *sweep, uint64_t *refine, void *stream)
+{
+    lfd_status s;
+    if ((s = need_bound(ctx)) != LFD_OK) return s;
+    if ((s = set_device(ctx)) != LFD_OK) return s;
+    LFD_CUDA(cudaStreamSynchronize((cudaStream_t)stream));
+    DevCounters h;
+    LFD_CUDA(cudaMemcpy(&h, ctx->d_ctr, sizeof(h), cudaMemcpyDeviceToHost));
+    if (sweep) *sweep = h.taken_sweep;
+    if (refine) *refine = h.taken_refine;
     return LFD_OK;
 }
 

@@ -81,6 +81,7 @@ struct PairDev {
 struct DevCounters {
     unsigned long long hyp;
     unsigned long long samples;
+    unsigned long long taken_sweep, taken_refine;   // samples the kernels took (lfd_samples_taken)
     int status;
     int bad_view, bad_index, pad;
 };

@@ -111,6 +111,7 @@ def load(build_if_missing: bool = True):
     lib.lfd_estimate_host.argtypes = [vp, P(LightFieldC), P(Params), P(vp), P(vp), vp]
     lib.lfd_synchronize.argtypes = [vp, vp]
     lib.lfd_counters.argtypes = [vp, P(C.c_uint64), P(C.c_uint64), vp]
+    lib.lfd_samples_taken.argtypes = [vp, P(C.c_uint64), P(C.c_uint64), vp]
     lib.lfd_score.argtypes = [vp, P(vp), i32, P(Query), P(C.c_float), vp]
     lib.lfd_get_superpixels.argtypes = [vp, i32, vp, vp, vp, vp, vp]
     lib.lfd_neighbor_views.argtypes = [P(Camera), i32, i32, P(i32), P(i32)]
@@ -146,7 +147,7 @@ def load(build_if_missing: bool = True):
     lib.lfd_server_import_state.argtypes = [vp, i32, vp, C.c_int64]
     for name in ("lfd_create", "lfd_destroy", "lfd_set_input", "lfd_num_superpixels", "lfd_plane_sweep",
                  "lfd_rasterize", "lfd_iterate", "lfd_estimate", "lfd_estimate_host", "lfd_synchronize",
-                 "lfd_counters", "lfd_score", "lfd_get_superpixels", "lfd_neighbor_views", "lfd_profile_enable",
+                 "lfd_counters", "lfd_samples_taken", "lfd_score", "lfd_get_superpixels", "lfd_neighbor_views", "lfd_profile_enable",
                  "lfd_profile_read", "lfd_estimate_batch", "lfd_estimate_batch_warm", "lfd_launch_config", "lfd_set_pair_forms", "lfd_pair_form", "lfd_workspace_required", "lfd_fuse", "lfd_slic",
                  "lfd_server_create", "lfd_server_destroy", "lfd_server_configure", "lfd_server_submit",
                  "lfd_server_poll", "lfd_server_export_state", "lfd_server_import_state", "lfd_server_set_max_batch",
@@ -555,6 +556,12 @@ class Context:
     def counters(self, stream=None):
         a, b = C.c_uint64(), C.c_uint64()
         self._check(self.lib.lfd_counters(self.h, C.byref(a), C.byref(b), _stream(stream)), "lfd_counters")
+        return int(a.value), int(b.value)
+
+    def samples_taken(self, stream=None):
+        """(sweep, refinement) samples taken to decide the hypotheses of `counters`."""
+        a, b = C.c_uint64(), C.c_uint64()
+        self._check(self.lib.lfd_samples_taken(self.h, C.byref(a), C.byref(b), _stream(stream)), "lfd_samples_taken")
         return int(a.value), int(b.value)
 
     STAGES = ("superpixels", "sweep", "raster", "propagate", "fusion")
