@@ -305,7 +305,9 @@ typedef struct {
                                   camera, parameter and option) is identical replays it, reading
                                   the current contents of the same image and label buffers.
                                   Needs a non-default stream. */
-    int32_t sweep_threads;     /* 128 or 256 (0 = 256): labels scored in parallel per superpixel */
+    int32_t sweep_threads;     /* 128 or 256 (0 = 256): labels scored in parallel per superpixel by a full
+                                  sweep; persistent sweeps of up to 256 labels drop labels that can no
+                                  longer win and use CTAs of 128 threads */
     int32_t sweep_persistent;  /* 1: persistent sweep CTAs take superpixels from a queue ordered
                                   by size (pixel-slot class ceil(n/32)), largest first */
     int32_t prop_blocks;       /* 7 or 8 (0 = 8) resident propagation CTAs per SM */

@@ -469,7 +469,7 @@ size_t workspace_need(const Layout &L, int fmt)
     add(4 * S); add(4 * (S + 1)); add(4 * S); add(4 * P);
     add(8 * S); add(16 * S); add(16 * S); add(32 * S); add(16 * S); add(16 * S);
     add(sizeof(DevCounters));
-    add(4 * S); add(4 * S); add(4 * ORDER_KEYS_HOST); add(64); add(sizeof(float *) * V);
+    add(4 * S); add(4 * S); add(4 * ORDER_KEYS_HOST); add(4 * QUEUE_INTS); add(sizeof(float *) * V);
     add(16 * S); add(16 * S); add(4 * S); add(8 * S); add(8 * S);
     for (int v = 0; v < V; v++) add((size_t)qb * (L.W[v] + 1) * (L.H[v] + 1));
     for (int v = 0; v < V; v++) add((size_t)16 * L.W[v] * L.H[v]);
@@ -872,12 +872,15 @@ lfd_status rasterize_state(lfd_ctx *ctx, const float4 *planes, float *const *dep
 lfd_status run_sweep(lfd_ctx *ctx, float *cost, cudaStream_t st)
 {
     if (ctx->lc.sweep_persistent) LFD_CUDA(cudaMemsetAsync(ctx->d_queue, 0, 4 * QUEUE_INTS, st));
+    int bounded = ctx->lc.sweep_persistent;
+    for (const LfInfo &l : ctx->lfs) bounded = bounded && l.p.num_labels <= SWEEP_BOUNDED_LABELS;
     for (int k = 0; k < NSCLASS; k++) {
         if (!ctx->cls_count[k]) continue;
         const int threads = std::min(LCLASS_THREADS[k / 3], ctx->lc.sweep_threads);
         Consts c = ctx->c;                   // the class's pair form
         c.affine = k % 3 >= 1;
         c.shift = k % 3 == 2;
+        c.sweep_bounded = bounded;
         LFD_CUDA(traced(ctx, LFD_STAGE_SWEEP, st, [&] {
             return launch_sweep(ctx->w, c, ctx->lc, threads, ctx->cls_base[k], ctx->cls_count[k], 4 + k,
                                 ctx->d_planesA, ctx->d_label, cost, st);

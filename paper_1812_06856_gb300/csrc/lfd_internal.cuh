@@ -92,6 +92,7 @@ struct Consts {
     int sweep_frame;
     int batch_iters;         // 1: a view whose light field has run its iterations passes its plane through
     float col_scale;         // sampler colour units -> [0,1]
+    int sweep_bounded;       // 1: a sweep without costs may drop labels that can no longer win (k_sweep_bounded)
     int cand_batch;          // candidate planes per pass (16 or 32; LaunchCfg::prop_batch)
     int affine;              // 1: every pair's homography has third row (0, 0, c) for every plane
                              //    (parallel cameras, common principal depth axis): the sample's depth
@@ -119,7 +120,7 @@ struct Workspace {
     DevCounters *ctr;
     const int *order;        // [S_total] work order: descending pixel-slot class, index order inside
     const int *order_sweep;  // [S_total] sweep work order: descending power-of-two size class, index order inside
-    int *queue;              // [32] work-queue counters of persistent launches
+    int *queue;              // [QUEUE_INTS] work-queue counters of persistent launches
     int S_total;
     long long px_total;
 };
@@ -280,6 +281,7 @@ constexpr int LCLASS_THREADS[LCLASSES] = {64, 128, 160, 192, 224, 256};
 // sweep classes: one sweep launch per (label-count class, pair form) present,
 // so that each view of a batch of mixed rigs sweeps with its own pair form
 constexpr int NSCLASS = LCLASSES * 3;
+constexpr int SWEEP_BOUNDED_LABELS = 256;   // labels of a bounded sweep (Consts::sweep_bounded); more: full sweep
 constexpr int QUEUE_INTS = 32;          // 4 + NSCLASS <= QUEUE_INTS
 inline int label_class(int L)
 {

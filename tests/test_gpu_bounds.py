@@ -95,3 +95,59 @@ def test_scan_order_does_not_change_the_choice(lfd, colour):
     for planes, depth, hyp, samples in out[1:]:
         assert torch.equal(planes, out[0][0]) and torch.equal(depth, out[0][1])
         assert (hyp, samples) == out[0][2:]
+
+
+def _views(kind, rig, fmt):
+    H, W, V = rig.H, rig.W, rig.V
+    if kind == "rendered":
+        scene = synth._random_scene(np.random.default_rng(2), 4, 1, 1, float(rig.K[0, 0, 0]), 2.0, 8.0, 1.8)
+        rgb, _, _ = synth.render(rig, scene, "cuda")
+    else:                      # "flat": every label costs the same; "steps": many labels tie, few differ
+        rgb = torch.full((V, H, W, 3), 0.25, dtype=torch.float64, device="cuda")
+        if kind == "steps":
+            rgb[:, :, W // 2:] = 0.75
+    if fmt == "rgba8":
+        return synth.quantize_rgba8(rgb)
+    dt = {"rgba_f16": torch.float16, "rgba_bf16": torch.bfloat16, "rgba_f32": torch.float32}[fmt]
+    v = synth.to_rgba_float(rgb, dt)
+    if kind == "rendered":     # a few texels without a finite colour
+        v[0, H // 2, W // 3, 0] = float("nan")
+        v[1, H // 3, W // 2, 1] = float("inf")
+    return v
+
+
+# label counts around a pass (32), the lane stage (48) and the bounded sweep's limit (256); pitches with
+# superpixels below a warp, around one chunk of 128 pixels, of several chunks, and above 4096 pixels
+@pytest.mark.parametrize("rig,fmt,form,L,pitch,kind", [
+    ("grid", "rgba_f16", 2, 256, 16, "rendered"), ("grid", "rgba8", 2, 255, 5, "rendered"),
+    ("grid", "rgba8", 1, 33, 11, "rendered"), ("arc", "rgba8", 0, 256, 14, "rendered"),
+    ("arc", "rgba_bf16", 0, 49, 23, "rendered"), ("arc", "rgba_f32", 0, 100, 12, "rendered"),
+    ("grid", "rgba_f32", 2, 64, 9, "rendered"), ("grid", "rgba_f32", 1, 48, 30, "rendered"),
+    ("pair", "rgba8", 2, 32, 8, "rendered"), ("pair", "rgba_f16", 2, 1, 16, "rendered"),
+    ("pair", "rgba_f16", 0, 2, 16, "rendered"), ("grid", "rgba8", 2, 257, 16, "rendered"),
+    ("grid", "rgba8", 2, 256, 16, "flat"), ("arc", "rgba8", 0, 200, 16, "flat"),
+    ("grid", "rgba8", 2, 256, 16, "steps"), ("arc", "rgba_f16", 0, 256, 20, "steps"),
+    ("grid", "rgba8", 2, 70, 90, "rendered"), ("arc", "rgba8", 0, 70, 300, "rendered"),
+])
+@pytest.mark.parametrize("T", [0.04, 1e-6, float("inf")])
+def test_bounded_sweep_picks_the_full_sweeps_label(lfd, rig, fmt, form, L, pitch, kind, T):
+    W, H = 301, 203
+    f = 300.0 * W / 320.0
+    r = {"grid": lambda: synth.grid_rig(2, 2, 0.08, f, W, H), "arc": lambda: synth.arc_rig(5, 30.0, 5.0, f, W, H),
+         "pair": lambda: synth.line_rig(2, 0.1, f, W, H)}[rig]()
+    views = _views(kind, r, fmt)
+    maps = [synth.grid_labels_fast(W, H, pitch, True, seed=v, device="cuda") for v in range(r.V)]
+    labels, (GW, GH) = torch.stack([m[0] for m in maps]).contiguous(), maps[0][1:]
+    ctx = lfd.Context(0)
+    ctx.set_pair_forms(form)
+    ctx.set_input(views, labels, r.K, r.R, r.t, GW, GH, dict(d_min=2.0, d_max=8.0, num_labels=L, T=T))
+    assert ctx.pair_form() == form
+    full_planes, full_labels, _ = ctx.plane_sweep(want_labels=True, want_costs=True)
+    taken_full = ctx.samples_taken()[0]
+    planes, lab, _ = ctx.plane_sweep(want_labels=True)
+    ctx.synchronize()
+    assert torch.equal(lab, full_labels)
+    assert torch.equal(planes, full_planes)
+    assert taken_full == L * r.V * W * H * (r.V - 1)
+    if kind == "rendered" and 64 <= L <= 256 and T == 0.04 and pitch < 60:
+        assert ctx.samples_taken()[0] - taken_full < 0.9 * taken_full      # labels were excluded
