@@ -283,8 +283,9 @@ lfd_status lfd_slic(lfd_ctx *ctx, int32_t n, const void *const *views, const int
  * the closest candidate with stability >= 0 is written (0 if none).
  *   depth_in / depth_out: host arrays [V] of device float[H*W] (the layout of
  *   lfd_estimate's depth maps); must not alias.  tau > 0 (0.01 = 1 %).
- * The z-buffers (V_l - 1 planes per view of the largest light field) are
- * allocated on first use outside the context's budget.  Asynchronous. */
+ * The z-buffers (V_l - 1 planes per reference view, for as many views at a
+ * time as fit 512 MB, at least one) are allocated on first use outside the
+ * context's budget.  Asynchronous. */
 lfd_status lfd_fuse(lfd_ctx *ctx, const float *const *depth_in, float *const *depth_out, double tau, void *stream);
 
 /* ---- batched frames --------------------------------------------------- */

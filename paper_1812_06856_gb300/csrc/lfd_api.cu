@@ -10,6 +10,7 @@
 #include <string>
 #include <vector>
 
+#include "lfd_fuse.cuh"
 #include "lfd_internal.cuh"
 #include "lfd_slic.cuh"
 
@@ -231,8 +232,9 @@ struct lfd_ctx {
     std::vector<lfd_camera> cams;    // cameras of the bound views (global order)
     void *d_slic = nullptr;          // SLIC scratch (CIELAB image, centres)
     size_t slic_cap = 0;
-    unsigned *d_zbuf = nullptr;      // fusion z-buffers (one light field at a time)
+    unsigned *d_zbuf = nullptr;      // fusion z-buffers (one group of reference views at a time)
     size_t zbuf_cap = 0;
+    bool zbuf_clean = false;         // every word is +inf once the enqueued work has run
     void *d_ftab = nullptr;
     size_t ftab_cap = 0;
     // CUDA graph of a batched frame and the pinned depth table it reads
@@ -1613,18 +1615,40 @@ lfd_status lfd_fuse(lfd_ctx *ctx, const float *const *depth_in, float *const *de
         if (depth_in[v] == depth_out[v]) return fail(ctx, LFD_ERR_INVALID_ARG, "view %d: depth_in aliases depth_out", v);
     }
     cudaStream_t st = (cudaStream_t)stream;
-    // z-buffer and table sizes: the largest light field
+    // groups of reference views whose z-buffers (words) fit FUSE_GROUP_BYTES; sizes for the largest
+    struct Group {
+        int first, count;
+    };
+    std::vector<std::vector<Group>> groups;
     size_t zmax = 0, tmax = 0;
     for (const LfInfo &l : ctx->lfs) {
         size_t z = 0;
-        for (int k = 0; k < l.V; k++) z += (size_t)(l.V - 1) * ctx->L.W[l.first_view + k] * ctx->L.H[l.first_view + k];
-        zmax = std::max(zmax, z);
+        groups.emplace_back();
+        for (int k = 0; k < l.V; k++) {
+            const size_t zk = (size_t)(l.V - 1) * ctx->L.W[l.first_view + k] * ctx->L.H[l.first_view + k];
+            if (k == 0 || 4 * (z + zk) > FUSE_GROUP_BYTES || groups.back().back().count == FUSE_MAX_GROUP) {
+                groups.back().push_back({k, 0});
+                z = 0;
+            }
+            groups.back().back().count++;
+            z += zk;
+            zmax = std::max(zmax, z);
+        }
         const size_t t = align_up(8 * (size_t)l.V, 16) + 8 * (size_t)l.V + 16 * (size_t)l.V + 48 * (size_t)l.V * l.V;
         tmax = std::max(tmax, t);
     }
-    if ((s = ensure_dev(ctx, (void **)&ctx->d_zbuf, &ctx->zbuf_cap, 4 * std::max<size_t>(zmax, 1))) != LFD_OK) return s;
+    const size_t zcap = ctx->zbuf_cap;
+    if ((s = ensure_dev(ctx, (void **)&ctx->d_zbuf, &ctx->zbuf_cap, align_up(4 * std::max<size_t>(zmax, 1), 16))) != LFD_OK)
+        return s;
     if ((s = ensure_dev(ctx, &ctx->d_ftab, &ctx->ftab_cap, tmax)) != LFD_OK) return s;
-    for (const LfInfo &l : ctx->lfs) {
+    // under capture nothing runs yet: the graph clears for itself and the next call clears again
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    const bool capturing = cudaStreamIsCapturing(st, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone;
+    if (ctx->zbuf_cap != zcap || !ctx->zbuf_clean || capturing)
+        LFD_CUDA(traced(ctx, LFD_STAGE_FUSION, st, [&] { return launch_fuse_clear(ctx->d_zbuf, ctx->zbuf_cap, st); }));
+    ctx->zbuf_clean = false;                 // until every group that is started below is enqueued
+    for (size_t li = 0; li < ctx->lfs.size(); li++) {
+        const LfInfo &l = ctx->lfs[li];
         const int V = l.V, f = l.first_view;
         // table: W, H (int), zoff (int64), depth_in, depth_out (pointers), mats (float)
         const size_t o_wh = 0, o_zoff = align_up(8 * (size_t)V, 16), o_in = o_zoff + 8 * (size_t)V,
@@ -1637,13 +1661,19 @@ lfd_status lfd_fuse(lfd_ctx *ctx, const float *const *depth_in, float *const *de
         const float **hin = (const float **)(h + o_in);
         float **hout = (float **)(h + o_out);
         float *hm = (float *)(h + o_mats);
-        long long zw = 0;
-        int max_px = 0;
+        int max_px = 0, max_w = 0, max_h = 0;
+        for (const Group &g : groups[li]) {
+            long long zw = 0;
+            for (int k = g.first; k < g.first + g.count; k++) {
+                hz[k] = zw;
+                zw += (long long)(V - 1) * ctx->L.W[f + k] * ctx->L.H[f + k];
+            }
+        }
         for (int k = 0; k < V; k++) {
             hw[k] = ctx->L.W[f + k];
             hh[k] = ctx->L.H[f + k];
-            hz[k] = zw;
-            zw += (long long)(V - 1) * hw[k] * hh[k];
+            max_w = std::max(max_w, hw[k]);
+            max_h = std::max(max_h, hh[k]);
             max_px = std::max(max_px, hw[k] * hh[k]);
             hin[k] = depth_in[f + k];
             hout[k] = depth_out[f + k];
@@ -1687,8 +1717,11 @@ lfd_status lfd_fuse(lfd_ctx *ctx, const float *const *depth_in, float *const *de
         a.depth_out = (float *const *)(d + o_out);
         a.mats = (const float *)(d + o_mats);
         a.zbuf = ctx->d_zbuf;
-        LFD_CUDA(traced(ctx, LFD_STAGE_FUSION, st, [&] { return launch_fuse(a, zw, max_px, st); }, 3));
+        for (const Group &g : groups[li])
+            LFD_CUDA(traced(ctx, LFD_STAGE_FUSION, st,
+                            [&] { return launch_fuse_group(a, g.first, g.count, max_w, max_h, max_px, st); }, 2));
     }
+    ctx->zbuf_clean = !capturing;
     return LFD_OK;
 }
 
