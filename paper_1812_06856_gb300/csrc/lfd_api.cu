@@ -1740,10 +1740,14 @@ lfd_status lfd_slic(lfd_ctx *ctx, int32_t n, const void *const *views, const int
         return fail(ctx, LFD_ERR_INVALID_ARG, "lfd_slic: bad arguments");
     if (!(compactness > 0.0) || iterations < 0 || iterations > 1000)
         return fail(ctx, LFD_ERR_INVALID_ARG, "compactness must be > 0 and iterations 0..1000");
+    auto cell_stride = [&](int v) {      // largest cell: edges at round(k size / n)
+        const size_t cw = (width[v] + grid_w[v] - 1) / grid_w[v], ch = (height[v] + grid_h[v] - 1) / grid_h[v];
+        return align_up(cw * ch, 4);
+    };
     auto view_bytes = [&](int v, size_t &o_c, size_t &sz_c) {
-        o_c = align_up(16 * (size_t)width[v] * height[v], 256);
+        o_c = align_up(16 * cell_stride(v) * grid_w[v] * grid_h[v], 256);
         sz_c = align_up(20 * (size_t)grid_w[v] * grid_h[v], 256);
-        return o_c + 2 * sz_c + align_up(48 * (size_t)grid_w[v] * grid_h[v], 256);
+        return o_c + 2 * sz_c + align_up(cell_stride(v) * grid_w[v] * grid_h[v], 256);
     };
     for (int v = 0; v < n; v++) {
         if (width[v] < 1 || height[v] < 1 || width[v] > LFD_MAX_DIM || height[v] > LFD_MAX_DIM || grid_w[v] < 1 ||
@@ -1776,19 +1780,20 @@ lfd_status lfd_slic(lfd_ctx *ctx, int32_t n, const void *const *views, const int
             sv.GW = grid_w[v];
             sv.GH = grid_h[v];
             sv.fmt = fmt;
-            sv.pad = 0;
+            sv.stride = (int)cell_stride(v);
             sv.pitch = view_pitch_bytes && view_pitch_bytes[v] ? view_pitch_bytes[v] : (long long)width[v] * tb;
             sv.img = views[v];
             sv.lab = (float4 *)base;
             sv.centres = (float *)(base + o_c);
             sv.centres2 = (float *)(base + o_c + sz_c);
-            sv.acc = (unsigned long long *)(base + o_c + 2 * sz_c);
+            sv.code = (unsigned char *)(base + o_c + 2 * sz_c);
             sv.labels = labels_out[v];
             base += bytes;
             const double step = std::sqrt((double)sv.W * sv.H / ((double)sv.GW * sv.GH));
             b.wxy[k] = (float)((compactness / step) * (compactness / step));
             b.max_px = std::max(b.max_px, sv.W * sv.H);
             b.max_cells = std::max(b.max_cells, sv.GW * sv.GH);
+            b.max_stride = std::max(b.max_stride, sv.stride);
         }
         LFD_CUDA(launch_slic(b, centres_in ? centres_in + g : nullptr, iterations, centres_out ? centres_out + g : nullptr,
                              st));

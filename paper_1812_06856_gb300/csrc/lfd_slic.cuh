@@ -8,13 +8,14 @@ namespace lfd {
 
 // one view of a SLIC segmentation
 struct SlicView {
-    int W, H, GW, GH, fmt, pad;
+    int W, H, GW, GH, fmt;
+    int stride;                      // entries of `lab` and `code` per cell (the largest cell, rounded up to 4)
     long long pitch;                 // bytes per image row
     const void *img;
-    float4 *lab;                     // [W*H] CIELAB of the view (scratch)
+    float4 *lab;                     // [GW*GH][stride] CIELAB and position of a cell's pixels (scratch)
+    unsigned char *code;             // [GW*GH][stride] the pixels' picks among the 3x3 cells (scratch)
     int *labels;                     // [W*H] output
     float *centres, *centres2;       // [GW*GH][5] {L, a, b, x, y} (scratch, ping-pong)
-    unsigned long long *acc;         // [GW*GH][6] update sums {L, a, b (fixed point), x, y, count} (scratch)
 };
 
 // up to SLIC_BATCH views segmented by the same launches (blockIdx.y = view)
@@ -22,7 +23,7 @@ constexpr int SLIC_BATCH = 16;
 struct SlicBatch {
     SlicView v[SLIC_BATCH];
     float wxy[SLIC_BATCH];                // (m / S)^2 of each view
-    int n, max_px, max_cells, pad;
+    int n, max_px, max_cells, max_stride;
 };
 
 cudaError_t launch_slic(const SlicBatch &b, const float *const *centres_in, int iterations,
