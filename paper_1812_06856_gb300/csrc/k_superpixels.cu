@@ -8,66 +8,54 @@
 // neighbours, which is fixed per superpixel and computed here once.
 //
 // The pixel lists are built without sorting and without atomics on the list
-// itself: one block per superpixel scans the superpixel's bounding box in
-// row-major order and compacts the matching pixels with a block prefix sum,
-// so the list order (row-major) and every sum are deterministic.  The cost is
-// the sum of bounding-box areas, about the image area for compact superpixels.
-#include "lfd_internal.cuh"
+// itself: one warp per superpixel (a CTA for large ones) scans the
+// superpixel's bounding box in row-major order and compacts the matching
+// pixels by ballots, so the list order (row-major) and every sum are
+// deterministic.  The cost is the sum of bounding-box areas, about the image
+// area for compact superpixels.
+#include "lfd_superpixels.cuh"
 
 namespace lfd {
 
 // ---------------------------------------------------------------------------
-// 1. counts and bounding boxes (warp-aggregated atomics)
+// 1. counts and bounding boxes (label_runs, lfd_superpixels.cuh)
 // ---------------------------------------------------------------------------
 
+// blockIdx.y = view; one warp per strip of 32 columns x SP_STRIP rows
 __global__ void __launch_bounds__(256) k_sp_count(Workspace w, int *cnt, int4 *bbox)
 {
     const int v = blockIdx.y;
     const ViewDev &vd = w.views[v];
-    const int npx = vd.W * vd.H;
-    const int p = blockIdx.x * blockDim.x + threadIdx.x;
-    const bool in = p < npx;
-    int l = in ? __ldg(vd.labels + p) : -1;
-    const bool ok = in && l >= 0 && l < vd.S;
-    if (in && !ok) {
-        if (atomicOr(&w.ctr->status, DEV_ERR_LABEL) == 0) {
-            w.ctr->bad_view = v;
-            w.ctr->bad_index = p;
-        }
-    }
-    const unsigned act = __ballot_sync(0xffffffffu, ok);
-    if (!ok) return;
-    const int x = p % vd.W, y = p / vd.W;
-    const unsigned grp = __match_any_sync(act, l);
-    const int n = __popc(grp);
-    const int mnx = (int)__reduce_min_sync(grp, (unsigned)x);
-    const int mxx = (int)__reduce_max_sync(grp, (unsigned)x);
-    const int mny = (int)__reduce_min_sync(grp, (unsigned)y);
-    const int mxy = (int)__reduce_max_sync(grp, (unsigned)y);
-    if ((threadIdx.x & 31) == __ffs(grp) - 1) {
-        const int gs = vd.sp_base + l;
-        atomicAdd(&cnt[gs], n);
-        atomicMin(&bbox[gs].x, mnx);
-        atomicMin(&bbox[gs].y, mny);
-        atomicMax(&bbox[gs].z, mxx);
-        atomicMax(&bbox[gs].w, mxy);
+    const int bad = label_runs(vd.labels, vd.W, vd.H, vd.S, cnt + vd.sp_base, bbox + vd.sp_base,
+                               blockIdx.x * 8 + (threadIdx.x >> 5));
+    if (bad >= 0 && atomicOr(&w.ctr->status, DEV_ERR_LABEL) == 0) {
+        w.ctr->bad_view = v;
+        w.ctr->bad_index = bad;
     }
 }
 
-__global__ void k_sp_bbox_init(int S_total, int *cnt, int4 *bbox)
+// per superpixel: empty count and box, and its view (the last one whose first
+// superpixel is not behind it)
+__global__ void k_sp_init(Workspace w, int V, int *cnt, int4 *bbox, int *sp_view)
 {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < S_total) {
-        cnt[i] = 0;
-        bbox[i] = make_int4(0x7fffffff, 0x7fffffff, -1, -1);
+    if (i >= w.S_total) return;
+    cnt[i] = 0;
+    bbox[i] = make_int4(0x7fffffff, 0x7fffffff, -1, -1);
+    int lo = 0, hi = V - 1;
+    while (lo < hi) {
+        const int mid = (lo + hi + 1) >> 1;
+        if (w.views[mid].sp_base <= i) lo = mid;
+        else hi = mid - 1;
     }
+    sp_view[i] = lo;
 }
 
-cudaError_t launch_sp_count(const Workspace &w, int V, int max_px, int *cnt, int4 *bbox, cudaStream_t st)
+cudaError_t launch_sp_count(const Workspace &w, int V, int max_strips, int *cnt, int4 *bbox, int *sp_view,
+                            cudaStream_t st)
 {
-    k_sp_bbox_init<<<(w.S_total + 255) / 256, 256, 0, st>>>(w.S_total, cnt, bbox);
-    dim3 grid((max_px + 255) / 256, V);
-    k_sp_count<<<grid, 256, 0, st>>>(w, cnt, bbox);
+    k_sp_init<<<(w.S_total + 255) / 256, 256, 0, st>>>(w, V, cnt, bbox, sp_view);
+    k_sp_count<<<dim3((max_strips + 7) / 8, V), 256, 0, st>>>(w, cnt, bbox);
     return cudaGetLastError();
 }
 
@@ -125,126 +113,115 @@ cudaError_t launch_sp_scan(const Workspace &w, int V, const int *cnt, int *off, 
 // 3. ordered compaction of each superpixel's pixels + centroid and colour sums
 // ---------------------------------------------------------------------------
 
-struct ColourSum {
-    double r, g, b;
-};
+// One warp per superpixel; a superpixel whose box exceeds SP_WARP_AREA pixels
+// is left to a second pass of whole CTAs over the same grid.
+//
+// 8 x 1024x768 RGBA8 (32120 superpixels of 14 x 14): 590 -> 63 us; one CTA of
+// 256 threads per superpixel spent its time in five block-wide trees of FP64
+// and 64-bit sums.  Latency-bound (label, then texel); the lists, labels and
+// texels are 38 MB, 6 us at the HBM rate.
+constexpr int SP_WARP_AREA = 4096;
 
-__device__ __forceinline__ void texel_rgb(int fmt, const void *img, long long pitch, int x, int y, double &r,
-                                          double &g, double &b)
-{
-    const char *row = (const char *)img + (long long)y * pitch;
-    if (fmt == LFD_RGBA8) {
-        const uchar4 t = ((const uchar4 *)row)[x];
-        r = t.x; g = t.y; b = t.z;                       // summed as integers, scaled once at the end
-    } else if (fmt == LFD_RGBA_F16) {
-        const __half *t = (const __half *)row + 4 * x;
-        r = __half2float(t[0]); g = __half2float(t[1]); b = __half2float(t[2]);
-    } else if (fmt == LFD_RGBA_BF16) {
-        const __nv_bfloat16 *t = (const __nv_bfloat16 *)row + 4 * x;
-        r = __bfloat162float(t[0]); g = __bfloat162float(t[1]); b = __bfloat162float(t[2]);
-    } else {
-        const float4 t = ((const float4 *)row)[x];
-        r = t.x; g = t.y; b = t.z;
-    }
-}
-
-template <typename T>
-__device__ __forceinline__ T block_sum256(T v, T *sh)
-{
-    // fixed tree over 256 threads: deterministic
-    sh[threadIdx.x] = v;
-    __syncthreads();
-    for (int o = 128; o > 0; o >>= 1) {
-        if (threadIdx.x < o) sh[threadIdx.x] = sh[threadIdx.x] + sh[threadIdx.x + o];
-        __syncthreads();
-    }
-    T r = sh[0];
-    __syncthreads();
-    return r;
-}
-
+template <int FMT>
 __global__ void __launch_bounds__(256) k_sp_collect(Workspace w, Consts c, const int4 *bbox, const int *cnt,
                                                     unsigned *pix, double2 *cen, int2 *ref, float4 *col)
 {
-    const int gs = blockIdx.x;
-    const int v = w.sp_view[gs];
-    const ViewDev &vd = w.views[v];
-    const int s = gs - vd.sp_base;
-    const int n = cnt[gs];
-    __shared__ int warp_cnt[8];
-    __shared__ double shd[256];
-    __shared__ long long shl[256];
-    if (n == 0) {
-        if (threadIdx.x == 0) {
-            cen[gs] = make_double2(0.0, 0.0);
-            ref[gs] = make_int2(0, 0);
-            col[gs] = make_float4(0.f, 0.f, 0.f, 1.f);
-        }
-        return;
-    }
-    const int4 bb = bbox[gs];
-    const int bw = bb.z - bb.x + 1, bh = bb.w - bb.y + 1;
-    const long long area = (long long)bw * bh;
-    const int base_off = w.sp_off[gs];
+    __shared__ SuperpixelSums<FMT> part[8];
+    __shared__ int wcnt[8];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    long long sx = 0, sy = 0;
-    double sr = 0, sg = 0, sb = 0;
-    int written = 0;
-    for (long long b0 = 0; b0 < area; b0 += 256) {
-        const long long i = b0 + threadIdx.x;
-        int x = 0, y = 0;
-        bool f = false;
-        if (i < area) {
-            x = bb.x + (int)(i % bw);
-            y = bb.y + (int)(i / bw);
-            f = __ldg(vd.labels + (long long)y * vd.W + x) == s;
+    auto finish = [&](int gs, const SuperpixelSums<FMT> &t, int n) {     // one lane
+        double cx, cy, r, g, b;
+        t.mean(n, cx, cy, r, g, b);
+        cen[gs] = make_double2(cx, cy);
+        ref[gs] = make_int2(__double2int_rn(cx), __double2int_rn(cy));
+        col[gs] = make_float4((float)r, (float)g, (float)b, 1.0f);
+    };
+    const int gs0 = blockIdx.x * 8, gs = gs0 + wid;
+    bool large = false;
+    if (gs < w.S_total) {
+        const int n = cnt[gs];
+        if (n == 0) {
+            if (lane == 0) {
+                cen[gs] = make_double2(0.0, 0.0);
+                ref[gs] = make_int2(0, 0);
+                col[gs] = make_float4(0.f, 0.f, 0.f, 1.f);
+            }
+        } else {
+            const int4 bb = bbox[gs];
+            large = (long long)(bb.z - bb.x + 1) * (bb.w - bb.y + 1) > SP_WARP_AREA;
+            if (!large) {
+                const ViewDev &vd = w.views[__ldg(w.sp_view + gs)];
+                SuperpixelSums<FMT> t;
+                const int got = scan_box<FMT, true>(vd.labels, vd.img, vd.pitch, vd.W, gs - vd.sp_base, bb, 0, 1, lane,
+                                                    pix + w.sp_off[gs], n, t);
+                t.reduce();
+                if (lane == 0) {
+                    part[wid] = t;
+                    if (got != n && atomicOr(&w.ctr->status, DEV_ERR_COUNT) == 0) {
+                        w.ctr->bad_view = __ldg(w.sp_view + gs);
+                        w.ctr->bad_index = gs - vd.sp_base;
+                    }
+                }
+            }
         }
-        const unsigned bal = __ballot_sync(0xffffffffu, f);
-        if (lane == 0) warp_cnt[wid] = __popc(bal);
-        __syncthreads();
-        int before = 0, tot = 0;
-#pragma unroll
-        for (int k = 0; k < 8; k++) {
-            const int cw = warp_cnt[k];
-            before += k < wid ? cw : 0;
-            tot += cw;
-        }
-        if (f) {
-            const int rank = before + __popc(bal & ((1u << lane) - 1u));
-            if (written + rank < n) pix[base_off + written + rank] = ((unsigned)y << 16) | (unsigned)x;
-            sx += x;
-            sy += y;
-            double r, g, b;
-            texel_rgb(c.fmt, vd.img, vd.pitch, x, y, r, g, b);
-            sr += r; sg += g; sb += b;
-        }
-        written += tot;
-        __syncthreads();
+        if (lane == 0) wcnt[wid] = large ? -1 : n;
+    } else if (lane == 0) {
+        wcnt[wid] = 0;
     }
-    const long long tx = block_sum256<long long>(sx, shl);
-    const long long ty = block_sum256<long long>(sy, shl);
-    const double tr = block_sum256<double>(sr, shd);
-    const double tg = block_sum256<double>(sg, shd);
-    const double tb = block_sum256<double>(sb, shd);
-    if (threadIdx.x == 0) {
-        if (written != n) {
-            if (atomicOr(&w.ctr->status, DEV_ERR_COUNT) == 0) {
+    const bool any_large = __syncthreads_or(large);
+    // the warps' means, one lane each: FP64 divisions once per CTA
+    if (threadIdx.x < 8 && wcnt[threadIdx.x] > 0) finish(gs0 + threadIdx.x, part[threadIdx.x], wcnt[threadIdx.x]);
+    if (!any_large) return;
+    for (int k = 0; k < 8; k++) {
+        __syncthreads();
+        if (wcnt[k] >= 0) continue;          // uniform
+        const int g = gs0 + k, n = cnt[g], v = __ldg(w.sp_view + g);
+        const ViewDev &vd = w.views[v];
+        const int s = g - vd.sp_base;
+        const int4 bb = bbox[g];
+        // rows of the box split between the warps; a warp's place in the list follows from the warps before it
+        const int rows = bb.w - bb.y + 1, per = (rows + 7) / 8;
+        const int4 mine = make_int4(bb.x, min(bb.y + wid * per, bb.w + 1), bb.z, min(bb.y + (wid + 1) * per - 1, bb.w));
+        __shared__ int start[9];
+        SuperpixelSums<FMT> t;
+        const int got = mine.w < mine.y ? 0 : scan_box<FMT, false>(vd.labels, vd.img, vd.pitch, vd.W, s, mine, 0, 1,
+                                                                   lane, nullptr, 0, t);
+        if (lane == 0) start[wid + 1] = got;
+        __syncthreads();
+        int before = 0, total = 0;
+        for (int q = 0; q < 8; q++) {
+            before += q < wid ? start[q + 1] : 0;
+            total += start[q + 1];
+        }
+        if (mine.w >= mine.y && before < n) {
+            SuperpixelSums<FMT> dummy;
+            scan_box<FMT, true>(vd.labels, vd.img, vd.pitch, vd.W, s, mine, 0, 1, lane, pix + w.sp_off[g] + before,
+                                n - before, dummy);
+        }
+        t.reduce();
+        if (lane == 0) part[wid] = t;
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            for (int q = 1; q < 8; q++) part[0].add(part[q]);
+            if (total != n && atomicOr(&w.ctr->status, DEV_ERR_COUNT) == 0) {
                 w.ctr->bad_view = v;
                 w.ctr->bad_index = s;
             }
+            finish(g, part[0], n);
         }
-        const double cx = (double)tx / n, cy = (double)ty / n;
-        cen[gs] = make_double2(cx, cy);
-        ref[gs] = make_int2(__double2int_rn(cx), __double2int_rn(cy));
-        const double sc = (c.fmt == LFD_RGBA8) ? 1.0 / 255.0 : 1.0;
-        col[gs] = make_float4((float)(tr * sc / n), (float)(tg * sc / n), (float)(tb * sc / n), 1.0f);
     }
 }
 
 cudaError_t launch_sp_collect(const Workspace &w, const Consts &c, const int4 *bbox, const int *cnt, unsigned *pix,
                               double2 *cen, int2 *ref, float4 *col, cudaStream_t st)
 {
-    k_sp_collect<<<w.S_total, 256, 0, st>>>(w, c, bbox, cnt, pix, cen, ref, col);
+    const int blocks = (w.S_total + 7) / 8;
+    switch (c.fmt) {
+    case LFD_RGBA8: k_sp_collect<LFD_RGBA8><<<blocks, 256, 0, st>>>(w, c, bbox, cnt, pix, cen, ref, col); break;
+    case LFD_RGBA_F16: k_sp_collect<LFD_RGBA_F16><<<blocks, 256, 0, st>>>(w, c, bbox, cnt, pix, cen, ref, col); break;
+    case LFD_RGBA_BF16: k_sp_collect<LFD_RGBA_BF16><<<blocks, 256, 0, st>>>(w, c, bbox, cnt, pix, cen, ref, col); break;
+    default: k_sp_collect<LFD_RGBA_F32><<<blocks, 256, 0, st>>>(w, c, bbox, cnt, pix, cen, ref, col); break;
+    }
     return cudaGetLastError();
 }
 
@@ -262,7 +239,9 @@ __global__ void k_sp_minw(Workspace w, Consts c, float4 *col)
     const int gx = s % vd.GW, gy = s / vd.GW;
     const float4 cs = col[gs];
     const double k_col = vd.k_col;   // log2(e) / (2 alpha^2): omega = 2^(-|dC|^2 k_col)
-    double best = 1.0;
+    // the smallest similarity 2^-x is that of the largest x: one exponential
+    // instead of eight (FP64; 8 x 1024x768: 18.6 -> 10 us)
+    double far = 0.0;
     bool any = false;
     for (int d = 0; d < 8; d++) {
         int dx, dy;
@@ -273,11 +252,11 @@ __global__ void k_sp_minw(Workspace w, Consts c, float4 *col)
         if (w.sp_cnt[j] == 0) continue;
         const float4 cj = col[j];
         const double dr = (double)cj.x - cs.x, dg = (double)cj.y - cs.y, db = (double)cj.z - cs.z;
-        const double om = exp2(-(dr * dr + dg * dg + db * db) * k_col);
-        if (!any || om < best) best = om;
+        const double q = (dr * dr + dg * dg + db * db) * k_col;
+        if (!any || q > far) far = q;
         any = true;
     }
-    col[gs].w = (float)(any ? best : 1.0);
+    col[gs].w = (float)(any ? exp2(-far) : 1.0);
 }
 
 cudaError_t launch_sp_minw(const Workspace &w, const Consts &c, float4 *col, cudaStream_t st)
@@ -393,68 +372,149 @@ __device__ __forceinline__ int order_key(const Workspace &w, int gs, int mode, i
     return (ORDER_CLASSES - 1 - min(cls, ORDER_CLASSES - 1)) * ORDER_BANDS + band;   // 0 = largest class, top band
 }
 
-__global__ void k_order_hist(Workspace w, int *hist, int mode, int bands, const int *in)
+// Three launches: per tile of ORDER_TILE superpixels a histogram of the keys
+// (hist[key][tile]), one exclusive scan of it (key-major: the tile's first
+// slot of each key), and the scatter, where a superpixel's slot is its tile's
+// start of the key + the count of equal keys before it in the tile.  Both
+// orders go through the same launches (blockIdx.y): 13 us on 8 x 1024x768,
+// where a walk of one CTA over all tiles took 75 us per order.
+struct OrderJob {
+    int *order;
+    int *hist;
+    const int *in;
+    int mode;
+};
+
+struct OrderJobs {
+    OrderJob j[2];
+};
+
+__global__ void __launch_bounds__(ORDER_TILE) k_order_hist(Workspace w, const __grid_constant__ OrderJobs jobs,
+                                                           int tiles, int bands)
 {
+    const OrderJob &q = jobs.j[blockIdx.y];
     __shared__ int h[ORDER_KEYS];
-    for (int k = threadIdx.x; k < ORDER_KEYS; k += blockDim.x) h[k] = 0;
+    for (int k = threadIdx.x; k < ORDER_KEYS; k += ORDER_TILE) h[k] = 0;
     __syncthreads();
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < w.S_total) atomicAdd(&h[order_key(w, in ? __ldg(in + i) : i, mode, bands)], 1);
+    const int i = blockIdx.x * ORDER_TILE + threadIdx.x;
+    if (i < w.S_total) atomicAdd(&h[order_key(w, q.in ? __ldg(q.in + i) : i, q.mode, bands)], 1);
     __syncthreads();
-    for (int k = threadIdx.x; k < ORDER_KEYS; k += blockDim.x)
-        if (h[k]) atomicAdd(&hist[k], h[k]);
+    for (int k = threadIdx.x; k < ORDER_KEYS; k += ORDER_TILE) q.hist[k * tiles + blockIdx.x] = h[k];
 }
 
-// one CTA of 1024 threads walks the superpixels in tiles of 1024; a
-// superpixel's slot is its key's start + the count of equal keys before it
-__global__ void __launch_bounds__(1024) k_order_scatter(Workspace w, const int *hist, int *order, int mode, int bands,
-                                                        const int *in)
+// exclusive scan of ORDER_KEYS * tiles counts by one CTA, a contiguous run per thread
+__global__ void __launch_bounds__(1024) k_order_scan(const __grid_constant__ OrderJobs jobs, int tiles)
 {
-    __shared__ int run[ORDER_KEYS];                  // running position per key
-    __shared__ int wcnt[32][ORDER_KEYS];             // per-warp counts of the tile
+    int *hist = jobs.j[blockIdx.y].hist;
+    __shared__ int warp_tot[32];
     const int t = threadIdx.x, lane = t & 31, wid = t >> 5;
-    if (t == 0) {
-        int acc = 0;
-        for (int k = 0; k < ORDER_KEYS; k++) {
-            run[k] = acc;
-            acc += hist[k];
-        }
+    const int total = ORDER_KEYS * tiles, per = (total + 1023) / 1024, first = t * per, last = min(first + per, total);
+    int sum = 0;
+    for (int i = first; i < last; i++) sum += hist[i];
+    int incl = sum;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int u = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += u;
     }
-    for (int base = 0; base < w.S_total; base += 1024) {
-        for (int i = t; i < 32 * ORDER_KEYS; i += 1024) wcnt[i / ORDER_KEYS][i % ORDER_KEYS] = 0;
-        __syncthreads();
-        const int pos = base + t;
-        const bool ok = pos < w.S_total;
-        const int gs = ok ? (in ? __ldg(in + pos) : pos) : 0;
-        const int key = ok ? order_key(w, gs, mode, bands) : ORDER_KEYS;   // out-of-range lanes: a key of their own
-        const unsigned same = __match_any_sync(0xffffffffu, key);
-        const int rank = __popc(same & ((1u << lane) - 1u));
-        if (ok && rank == 0) wcnt[wid][key] = __popc(same);
-        __syncthreads();
-        if (ok) {
-            int before = 0;
-            for (int u = 0; u < wid; u++) before += wcnt[u][key];
-            order[run[key] + before + rank] = gs;
+    if (lane == 31) warp_tot[wid] = incl;
+    __syncthreads();
+    if (wid == 0) {
+        const int x = warp_tot[lane];
+        int y = x;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int u = __shfl_up_sync(0xffffffffu, y, o);
+            if (lane >= o) y += u;
         }
-        __syncthreads();
-        if (t < ORDER_KEYS) {
-            int tot = 0;
-            for (int u = 0; u < 32; u++) tot += wcnt[u][t];
-            run[t] += tot;
-        }
-        __syncthreads();
+        warp_tot[lane] = y - x;
+    }
+    __syncthreads();
+    int run = warp_tot[wid] + incl - sum;
+    for (int i = first; i < last; i++) {
+        const int x = hist[i];
+        hist[i] = run;
+        run += x;
     }
 }
 
-cudaError_t launch_sp_order(const Workspace &w, int *order, int *hist, int mode, int bands, const int *in,
-                            cudaStream_t st)
+__global__ void __launch_bounds__(ORDER_TILE) k_order_scatter(Workspace w, const __grid_constant__ OrderJobs jobs,
+                                                              int tiles, int bands)
+{
+    const OrderJob &q = jobs.j[blockIdx.y];
+    __shared__ unsigned short wcnt[ORDER_TILE / 32][ORDER_KEYS];     // per-warp counts of the tile
+    const int t = threadIdx.x, lane = t & 31, wid = t >> 5;
+    for (int i = t; i < (ORDER_TILE / 32) * ORDER_KEYS / 2; i += ORDER_TILE) ((unsigned *)wcnt)[i] = 0u;
+    __syncthreads();
+    const int pos = blockIdx.x * ORDER_TILE + t;
+    const bool ok = pos < w.S_total;
+    const int gs = ok ? (q.in ? __ldg(q.in + pos) : pos) : 0;
+    const int key = ok ? order_key(w, gs, q.mode, bands) : ORDER_KEYS;   // out-of-range lanes: a key of their own
+    const unsigned same = __match_any_sync(0xffffffffu, key);
+    const int rank = __popc(same & ((1u << lane) - 1u));
+    if (ok && rank == 0) wcnt[wid][key] = (unsigned short)__popc(same);
+    __syncthreads();
+    if (!ok) return;
+    int before = 0;
+    for (int u = 0; u < wid; u++) before += wcnt[u][key];
+    q.order[q.hist[key * tiles + blockIdx.x] + before + rank] = gs;
+}
+
+// up to one tile of superpixels: the whole sort in one CTA per order
+__global__ void __launch_bounds__(ORDER_TILE) k_order_small(Workspace w, const __grid_constant__ OrderJobs jobs,
+                                                            int bands)
+{
+    const OrderJob &q = jobs.j[blockIdx.y];
+    __shared__ unsigned short wcnt[ORDER_TILE / 32][ORDER_KEYS];
+    __shared__ int start[ORDER_TILE];
+    __shared__ int warp_tot[ORDER_TILE / 32];
+    const int t = threadIdx.x, lane = t & 31, wid = t >> 5;
+    for (int i = t; i < (ORDER_TILE / 32) * ORDER_KEYS / 2; i += ORDER_TILE) ((unsigned *)wcnt)[i] = 0u;
+    __syncthreads();
+    const bool ok = t < w.S_total;
+    const int gs = ok ? (q.in ? __ldg(q.in + t) : t) : 0;
+    const int key = ok ? order_key(w, gs, q.mode, bands) : ORDER_KEYS;
+    const unsigned same = __match_any_sync(0xffffffffu, key);
+    const int rank = __popc(same & ((1u << lane) - 1u));
+    if (ok && rank == 0) wcnt[wid][key] = (unsigned short)__popc(same);
+    __syncthreads();
+    // exclusive scan of the keys' totals, thread t = key t
+    int total = 0;
+    if (t < ORDER_KEYS)
+        for (int u = 0; u < ORDER_TILE / 32; u++) total += wcnt[u][t];
+    int incl = total;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int u = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += u;
+    }
+    if (lane == 31) warp_tot[wid] = incl;
+    __syncthreads();
+    int before = 0;
+    for (int u = 0; u < wid; u++) before += warp_tot[u];
+    start[t] = before + incl - total;
+    __syncthreads();
+    if (!ok) return;
+    before = start[key];
+    for (int u = 0; u < wid; u++) before += wcnt[u][key];
+    q.order[before + rank] = gs;
+}
+
+int order_kernels(int S_total) { return order_tiles(S_total) > 1 ? 3 : 1; }
+
+cudaError_t launch_sp_orders(const Workspace &w, int n, const SuperpixelOrder *o, int bands, cudaStream_t st)
 {
     bands = max(1, min(bands, ORDER_BANDS));
-    cudaError_t e = cudaMemsetAsync(hist, 0, sizeof(int) * ORDER_KEYS, st);
-    if (e != cudaSuccess) return e;
-    const int blocks = (w.S_total + 255) / 256;
-    k_order_hist<<<blocks, 256, 0, st>>>(w, hist, mode, bands, in);
-    k_order_scatter<<<1, 1024, 0, st>>>(w, hist, order, mode, bands, in);
+    const int tiles = order_tiles(w.S_total);
+    OrderJobs jobs = {};
+    for (int k = 0; k < n; k++) jobs.j[k] = {o[k].order, o[k].hist, o[k].in, o[k].mode};
+    if (tiles <= 1) {
+        k_order_small<<<dim3(1, n), ORDER_TILE, 0, st>>>(w, jobs, bands);
+        return cudaGetLastError();
+    }
+    k_order_hist<<<dim3(tiles, n), ORDER_TILE, 0, st>>>(w, jobs, tiles, bands);
+    k_order_scan<<<dim3(1, n), 1024, 0, st>>>(jobs, tiles);
+    k_order_scatter<<<dim3(tiles, n), ORDER_TILE, 0, st>>>(w, jobs, tiles, bands);
     return cudaGetLastError();
 }
 

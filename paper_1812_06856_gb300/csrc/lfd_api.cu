@@ -13,6 +13,7 @@
 #include "lfd_fuse.cuh"
 #include "lfd_internal.cuh"
 #include "lfd_slic.cuh"
+#include "lfd_superpixels.cuh"
 
 using namespace lfd;
 
@@ -203,7 +204,7 @@ struct lfd_ctx {
     short *d_radii = nullptr;
     int *d_radii_cnt = nullptr;
     DevCounters *d_ctr = nullptr;
-    int *d_order = nullptr, *d_order_sweep = nullptr, *d_hist = nullptr, *d_queue = nullptr;
+    int *d_order = nullptr, *d_order_sweep = nullptr, *d_queue = nullptr;
     float **d_depth_ptrs = nullptr;
     float4 *d_planesA = nullptr, *d_planesB = nullptr;
     int *d_label = nullptr, *d_choice = nullptr;
@@ -429,7 +430,6 @@ cudaError_t traced(lfd_ctx *ctx, int stage, cudaStream_t st, F launch, int kerne
 }
 
 // -- layout + workspace allocation -------------------------------------------
-constexpr int ORDER_KEYS_HOST = ORDER_KEYS;   // keys of the work orders' counting sort
 
 // Sizes of the bound views in call order (global numbering).
 lfd_status make_layout(lfd_ctx *ctx, int n, const lfd_lightfield *lfs, Layout &L)
@@ -471,7 +471,7 @@ size_t workspace_need(const Layout &L, int fmt)
     add(4 * S); add(4 * (S + 1)); add(4 * S); add(4 * P);
     add(8 * S); add(16 * S); add(16 * S); add(32 * S); add(16 * S); add(16 * S);
     add(sizeof(DevCounters));
-    add(4 * S); add(4 * S); add(4 * ORDER_KEYS_HOST); add(4 * QUEUE_INTS); add(sizeof(float *) * V);
+    add(4 * S); add(4 * S); add(4 * QUEUE_INTS); add(sizeof(float *) * V);
     add(16 * S); add(16 * S); add(4 * S); add(8 * S); add(8 * S);
     for (int v = 0; v < V; v++) add((size_t)qb * (L.W[v] + 1) * (L.H[v] + 1));
     for (int v = 0; v < V; v++) add((size_t)16 * L.W[v] * L.H[v]);
@@ -531,7 +531,6 @@ lfd_status plan_workspace(lfd_ctx *ctx, int n, const lfd_lightfield *lfs)
     ctx->d_ctr = (DevCounters *)a.take(sizeof(DevCounters));
     ctx->d_order = (int *)a.take(4 * S);
     ctx->d_order_sweep = (int *)a.take(4 * S);
-    ctx->d_hist = (int *)a.take(4 * ORDER_KEYS_HOST);
     ctx->d_queue = (int *)a.take(4 * QUEUE_INTS);
     ctx->d_depth_ptrs = (float **)a.take(sizeof(float *) * V);
     ctx->d_planesA = (float4 *)a.take(16 * S);
@@ -565,12 +564,6 @@ lfd_status plan_workspace(lfd_ctx *ctx, int n, const lfd_lightfield *lfs)
     w.S_total = L.S_total;
     w.px_total = L.px_total;
     return LFD_OK;
-}
-
-__global__ void k_fill_sp_view(int *sp_view, int base, int S, int v)
-{
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < S) sp_view[base + i] = v;
 }
 
 // Host half of binding n light fields: validation, workspace, records staged in
@@ -742,21 +735,22 @@ lfd_status build_orders(lfd_ctx *ctx, cudaStream_t st)
     const int bands = ctx->lc.order_bands;
     int classes = 0;
     for (int k = 0; k < NSCLASS; k++) classes += ctx->cls_count[k] > 0;
+    // histograms of several tiles (more than 1024 superpixels): 2176 bytes per
+    // tile for both, in the energy buffer (8 B per superpixel), which only
+    // lfd_iterate writes
+    int *hist = (int *)ctx->d_energy, *hist2 = hist + ORDER_KEYS * order_tiles(ctx->L.S_total);
+    const int kernels = order_kernels(ctx->L.S_total);
+    const SuperpixelOrder prop = {ctx->d_order, hist, nullptr, 0};
     if (classes > 1) {
-        LFD_CUDA(traced(ctx, LFD_STAGE_SUPERPIXELS, st, [&] {
-            return launch_sp_order(ctx->w, ctx->d_order, ctx->d_hist, 1, bands, nullptr, st);
-        }, 2));
-        LFD_CUDA(traced(ctx, LFD_STAGE_SUPERPIXELS, st, [&] {
-            return launch_sp_order(ctx->w, ctx->d_order_sweep, ctx->d_hist, 2, bands, ctx->d_order, st);
-        }, 2));
-    } else {
-        LFD_CUDA(traced(ctx, LFD_STAGE_SUPERPIXELS, st, [&] {
-            return launch_sp_order(ctx->w, ctx->d_order_sweep, ctx->d_hist, 1, bands, nullptr, st);
-        }, 2));
+        const SuperpixelOrder by_size = {ctx->d_order, hist, nullptr, 1},
+                              by_class = {ctx->d_order_sweep, hist, ctx->d_order, 2};
+        LFD_CUDA(traced(ctx, LFD_STAGE_SUPERPIXELS, st, [&] { return launch_sp_orders(ctx->w, 1, &by_size, bands, st); }, kernels));
+        LFD_CUDA(traced(ctx, LFD_STAGE_SUPERPIXELS, st, [&] { return launch_sp_orders(ctx->w, 1, &by_class, bands, st); }, kernels));
+        LFD_CUDA(traced(ctx, LFD_STAGE_SUPERPIXELS, st, [&] { return launch_sp_orders(ctx->w, 1, &prop, bands, st); }, kernels));
+        return LFD_OK;
     }
-    LFD_CUDA(traced(ctx, LFD_STAGE_SUPERPIXELS, st, [&] {
-        return launch_sp_order(ctx->w, ctx->d_order, ctx->d_hist, 0, bands, nullptr, st);
-    }, 2));
+    const SuperpixelOrder both[2] = {prop, {ctx->d_order_sweep, hist2, nullptr, 1}};
+    LFD_CUDA(traced(ctx, LFD_STAGE_SUPERPIXELS, st, [&] { return launch_sp_orders(ctx->w, 2, both, bands, st); }, kernels));
     return LFD_OK;
 }
 
@@ -770,14 +764,10 @@ lfd_status enqueue_input(lfd_ctx *ctx, cudaStream_t st, bool record_event)
     LFD_CUDA(cudaMemcpyAsync(ctx->d_views, ctx->stage.buf(), total, cudaMemcpyHostToDevice, st));
     if (record_event) LFD_CUDA(cudaEventRecord(ctx->stage.event(), st));
     LFD_CUDA(cudaMemsetAsync(ctx->d_ctr, 0, sizeof(DevCounters), st));
-    for (int v = 0; v < V; v++) {
-        LFD_CUDA(traced(ctx, LFD_STAGE_SUPERPIXELS, st, [&] {
-            k_fill_sp_view<<<(L.S[v] + 255) / 256, 256, 0, st>>>(ctx->d_sp_view, L.sp_base[v], L.S[v], v);
-            return cudaGetLastError();
-        }));
-    }
+    int max_strips = 0;
+    for (int v = 0; v < V; v++) max_strips = std::max(max_strips, label_strips(L.W[v], L.H[v]));
     LFD_CUDA(traced(ctx, LFD_STAGE_SUPERPIXELS, st, [&] {
-        return launch_sp_count(ctx->w, V, L.max_px, ctx->d_sp_cnt, ctx->d_bbox, st);
+        return launch_sp_count(ctx->w, V, max_strips, ctx->d_sp_cnt, ctx->d_bbox, ctx->d_sp_view, st);
     }, 2));
     LFD_CUDA(traced(ctx, LFD_STAGE_SUPERPIXELS, st,
                     [&] { return launch_sp_scan(ctx->w, V, ctx->d_sp_cnt, ctx->d_sp_off, st); }));
