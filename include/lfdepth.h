@@ -296,11 +296,11 @@ lfd_status lfd_fuse(lfd_ctx *ctx, const float *const *depth_in, float *const *de
 typedef struct {
     int32_t autotune;          /* 1: the first call with a new argument signature times, on its
                                   own input, the sweep (128/256 threads x grid/persistent x
-                                  1/16 row bands in the work order) and the propagation (7/8
-                                  CTAs per SM x grid/persistent warps/cooperative CTAs x 16/32
-                                  candidates per batch x 1/16 row bands, timed on the first and
-                                  the last iteration) and keeps the fastest of each; the shape
-                                  fields are then ignored */
+                                  1/16 row bands in the work order) and the propagation
+                                  (grid/persistent warps/cooperative CTAs x 16/32 candidates per
+                                  batch x 1/16 row bands, timed on the first and the last
+                                  iteration) and keeps the fastest of each; the shape fields are
+                                  then ignored */
     int32_t graph;             /* 1: the frame's device work is captured as a CUDA graph on the
                                   first call; a later call whose signature (every pointer, size,
                                   camera, parameter and option) is identical replays it, reading
@@ -311,18 +311,17 @@ typedef struct {
                                   longer win and use CTAs of 128 threads */
     int32_t sweep_persistent;  /* 1: persistent sweep CTAs take superpixels from a queue ordered
                                   by size (pixel-slot class ceil(n/32)), largest first */
-    int32_t prop_blocks;       /* 7 or 8 (0 = 8) resident propagation CTAs per SM */
+    int32_t prop_blocks;       /* 7 or 8 (0 = 8); both run 7 resident propagation CTAs per SM, the
+                                  faster register budget */
     int32_t prop_persistent;   /* 1: persistent propagation warps over the same ordered queue */
-    int32_t prop_batch;        /* 16 or 32 (0 = 32): candidate planes a warp scores per pass over the
-                                  neighbour views (their footprints share L1 across the pass) */
+    int32_t prop_batch;        /* 16 or 32 (0 = 32): candidate planes a warp prepares and ranks at a time */
     int32_t order_bands;       /* 1 or 16 (0 = 16): row bands of the work orders inside a size class
                                   (16: the superpixels in flight cover the same rows of every view) */
     int32_t prop_coop;         /* 1 (with prop_persistent): the 4 warps of a propagation CTA update
-                                  one superpixel together, its candidates split between them, so
-                                  they gather from one footprint per neighbour view (L1 reuse);
-                                  0: one superpixel per warp.  Same results either way; on the
-                                  16 x 1080p and 8 x 1024x768 frames 0 is faster (the kernel is
-                                  issue-bound and the split costs instructions and barriers). */
+                                  one superpixel together, its candidates split between them; 0: one
+                                  superpixel per warp, except that a last, partly filled wave of a
+                                  small input goes to whole CTAs.  Same results either way; on the
+                                  16 x 1080p and 8 x 1024x768 frames 0 is faster. */
 } lfd_batch_options;
 
 void lfd_batch_options_default(lfd_batch_options *o);

@@ -17,12 +17,14 @@
 //       the pixels whose 3-D point is not behind view i's surface, and O_i
 //       (Eq. 11) = eta (1 - min_j omega) when some pixel lies behind it.
 //
-// Mapping: one warp per superpixel; lanes own pixels (ceil(n/32) slots per
-// lane, a compile-time count chosen per superpixel, up to 10 staged in shared
-// memory and more streamed), so the gathers of a warp into a neighbour view's
-// map fall in a compact footprint.  Hypotheses are scored one after another by
-// the whole warp; per view the five sums are reduced with REDUX (counts) and
-// butterfly shuffles (sums) in a fixed order, so results are deterministic.
+// Mapping: one warp per superpixel (a CTA's four share one where superpixels
+// are few, single_warp_count); lanes own pixels (ceil(n/32) slots per lane, up
+// to 10 staged in shared memory and more streamed), so the gathers of a warp
+// into a neighbour view's map fall in a compact footprint.  Hypotheses are
+// scored one after another by the whole warp; per view the sums are reduced
+// with REDUX (counts) and butterfly shuffles in a fixed order, so results are
+// deterministic.  Views in which the whole superpixel lands inside the image
+// take a shorter sample without tests (view_term_inside).
 // A hypothesis is dropped as soon as an upper bound of its energy is below the
 // best energy found (best_of_batch): the choice is the one of the full sums.
 // What does not depend on the view (the FP32 form of the plane and E_s) is
@@ -41,6 +43,10 @@ namespace lfd {
 typedef double4_32a dbl4;
 
 constexpr int PROP_WARPS = 4;
+// resident CTAs per SM: 72 registers.  With 64 (8 CTAs) the gathers of fewer
+// samples are in flight: 8 x 1024x768 arc 12.1 -> 13.0 ms of propagation, two
+// warm rigs 10.1 -> 10.7, 16 x 1080p 55.2 -> 56.2; with 80 (6 CTAs) 12.6, 11.1, 65.9
+constexpr int PROP_CTAS = 7;
 constexpr int SLOTS_MAX = 10;   // pixel slots per lane staged in shared memory (320 pixels per warp)
 
 
@@ -132,8 +138,8 @@ cudaError_t launch_plane_prep(const Workspace &w, const Consts &c, const float4 
 // ---------------------------------------------------------------------------
 //
 // The map holds the superpixel's mean colour times sqrt(k_col) and the depth
-// value (inverse depth, or depth in the metric domain) times sqrt(k_sig) of
-// the view's light field, so that the exponents of Eq. 7 / Eq. 9 and of the
+// value (inverse depth, or depth in the metric domain; NaN where there is
+// none) times sqrt(k_sig) of the view's light field, so that the exponents of Eq. 7 / Eq. 9 and of the
 // Gaussian of Eq. 10 are plain squared distances in the energy kernel.  (An
 // 8-B texel {depth value, superpixel} with the colours in a table halves the
 // gathered bytes but adds a dependent gather per sample: measured 17-19 %
@@ -162,7 +168,8 @@ __global__ void __launch_bounds__(128) k_rasterize(Workspace w, Consts c, float 
         const bool ok = rc.w != 0.f && inv > 0.f && isfinite(inv);
         const float dv = ok ? (c.domain == 0 ? inv : 1.0f / inv) : 0.f;
         const long long p = (long long)y * vd.W + x;
-        map[p] = make_float4(cc.x, cc.y, cc.z, dv * dgain);
+        const float tw = dv * dgain;
+        map[p] = make_float4(cc.x, cc.y, cc.z, tw > 0.f ? tw : __int_as_float(0x7fffffff));
         if (dep) dep[p] = ok ? 1.0f / inv : 0.f;
     }
 }
@@ -233,6 +240,7 @@ struct alignas(16) SpShared {
     int best_m;
     float k_sig, xy_lo, xy_hi, eta;              // energy constants of the superpixel's light field
     float rdx, rdy;                              // ref - c (anchor pixel minus centroid)
+    float bx0, bx1, by0, by1;                    // box of the pixel offsets from ref (view_inside)
     float vmax, rnnb;                            // bound of V_i + O_i, 1 / number of neighbour views (cand_bound)
     int term_mask;
 };
@@ -255,8 +263,8 @@ struct alignas(16) CandShared {
 __shared__ SpShared g_sh[PROP_WARPS];
 __shared__ CandShared g_cs[PROP_WARPS];
 
-// Cooperative propagation (k_propagate_coop): the CTA's 4 warps refine one
-// superpixel together, so its record is per CTA; each warp keeps its own
+// Cooperative propagation: the CTA's 4 warps refine one superpixel together,
+// so its record is per CTA (the first warp's); each warp keeps its own
 // candidate batch.  The winners of the warps and the candidate index of
 // every batch slot meet in CoopShared.
 struct CoopShared {
@@ -269,15 +277,13 @@ struct CoopShared {
     float nx[PROP_WARPS], ny[PROP_WARPS], nz[PROP_WARPS];
     unsigned nh[PROP_WARPS], nv[PROP_WARPS];   // hypotheses scored and (candidate, view) pairs summed per warp
 };
-__shared__ SpShared g_shc[1];
 __shared__ CoopShared g_co;
 
 // the superpixel record of this warp: its own, or the CTA's in the cooperative form
 template <bool COOP>
 __device__ __forceinline__ SpShared &sp_shared()
 {
-    if constexpr (COOP) return g_shc[0];
-    else return g_sh[threadIdx.x >> 5];
+    return g_sh[COOP ? 0 : threadIdx.x >> 5];
 }
 
 struct Acc {
@@ -418,18 +424,31 @@ __device__ __forceinline__ void energy_sample(const ViewK &K, bool act, float du
                               cb, a);
 }
 
-// The view terms S_i, V_i, O_i (Eq. 9-11) of hypothesis h in neighbour view k,
-// identical in every lane.  SL pixel slots per lane; unless MASK_ALL, every
-// slot but the last is full (n > 32 (SL - 1)).
+// slots per lane that a superpixel of n pixels is summed with
+__device__ __forceinline__ int slot_class(int n)
+{
+    const int s = (n + 31) >> 5;
+    return s <= 1 ? 1 : (s <= 8 ? s : SLOTS_MAX);
+}
+
+// The view terms S_i, V_i, O_i (Eq. 9-11) of a hypothesis in one neighbour
+// view, identical in every lane.
 struct ViewTerms {
     float Si, Vi, Oi;
     unsigned cnt, nx, ny;
 };
 
-template <int DOMAIN, int SL, bool MASK_ALL, bool AFF>
-__device__ __forceinline__ ViewTerms view_term(const Workspace &w, const SpShared &sh, const WarpSP &S, const HypF &h,
-                                               int k, int lane)
+// View k of hypothesis h, whatever its pixels do there:
+// `slots` pixel slots per lane, every slot but the last taken as full unless
+// mask_all (n > 32 (slots - 1)).  One rolled loop for every slot count: it
+// serves the views that a superpixel's box straddles (and the scorer), and a
+// body per slot count next to view_term_inside's thrashes the instruction
+// cache (8 x 1024x768 arc: propagation 17.3 ms with unrolled bodies).
+template <int DOMAIN, bool AFF>
+__device__ __forceinline__ ViewTerms view_term(const Workspace &w, const SpShared &sh, const HypF &h, int k, int lane,
+                                               int slots, bool mask_all)
 {
+    const WarpSP &S = sh.S;
     const SpView &sv = sh.view[k];
     ViewK K;
     K.hw = fmaf(sv.qw, h.dgr, sv.hw_a);
@@ -444,36 +463,36 @@ __device__ __forceinline__ ViewTerms view_term(const Workspace &w, const SpShare
     K.xa_m = sv.xa_m; K.ya_m = sv.ya_m; K.Wi = sv.Wi; K.Hi = sv.Hi;
     K.map = sv.map;
     K.xy = DOMAIN == 0 ? sh.xy_lo : sh.xy_hi;
+    const float cr = S.cr, cg = S.cg, cb = S.cb;
+    const int n = S.n;
     Acc a = {0u, 0u, 0u, 0.f, 0.f};
     // affine pair: one reciprocal for every pixel; a plane behind
     // camera i there (hw <= 0) has no valid pixel
     const float r_aff = AFF ? rcp_approx(K.hw) : 0.f;
     if (!AFF || K.hw > 0.f) {
-        // slots j and j + 1 come from one shared-memory load; every slot
-        // but the last is full unless MASK_ALL
-#pragma unroll
-        for (int jp = 0; jp < (SL + 1) / 2; jp++) {
-            const int j0 = 2 * jp, j1 = 2 * jp + 1;
-            const float4 d = sh.px4[32 * jp + lane];
-            energy_sample<DOMAIN, AFF>(K, (!MASK_ALL && j0 + 1 < SL) || lane + 32 * j0 < S.n, d.x, d.z,
-                                       fmaf(h.g0, d.x, fmaf(h.g1, d.z, h.gr)), S.cr, S.cg, S.cb, a, r_aff);
-            if (j1 < SL)
-                energy_sample<DOMAIN, AFF>(K, (!MASK_ALL && j1 + 1 < SL) || lane + 32 * j1 < S.n, d.y, d.w,
-                                           fmaf(h.g0, d.y, fmaf(h.g1, d.w, h.gr)), S.cr, S.cg, S.cb, a, r_aff);
+        // slots j and j + 1 come from one shared-memory load
+#pragma unroll 1
+        for (int j = 0; j < slots; j += 2) {
+            const float4 d = sh.px4[16 * j + lane];
+            energy_sample<DOMAIN, AFF>(K, (!mask_all && j + 1 < slots) || lane + 32 * j < n, d.x, d.z,
+                                       fmaf(h.g0, d.x, fmaf(h.g1, d.z, h.gr)), cr, cg, cb, a, r_aff);
+            energy_sample<DOMAIN, AFF>(K, j + 1 < slots && ((!mask_all && j + 2 < slots) || lane + 32 * (j + 1) < n),
+                                       d.y, d.w, fmaf(h.g0, d.y, fmaf(h.g1, d.w, h.gr)), cr, cg, cb, a, r_aff);
         }
-        if (SL == SLOTS_MAX) {
-#pragma unroll 2
-            for (int i = 32 * SL + lane; i < S.n; i += 32) {    // pixels beyond the staged slots
+        if (slots == SLOTS_MAX) {
+#pragma unroll 1
+            for (int i = 32 * SLOTS_MAX + lane; i < n; i += 32) {    // pixels beyond the staged slots
                 const unsigned pk = __ldg(w.sp_pix + S.off + i);
                 const float du = (float)((int)(pk & 0xffff) - S.ref.x);
                 const float dv = (float)((int)(pk >> 16) - S.ref.y);
-                energy_sample<DOMAIN, AFF>(K, true, du, dv, fmaf(h.g0, du, fmaf(h.g1, dv, h.gr)), S.cr, S.cg, S.cb, a,
+                energy_sample<DOMAIN, AFF>(K, true, du, dv, fmaf(h.g0, du, fmaf(h.g1, dv, h.gr)), cr, cg, cb, a,
                                            r_aff);
             }
         }
     }
+    __syncwarp();
     ViewTerms t;
-    if (S.n < 65536) {    // counts fit 16 bits: one REDUX for |Omega_i| and |X_i|
+    if (n < 65536) {    // counts fit 16 bits: one REDUX for |Omega_i| and |X_i|
         const unsigned cx2 = __reduce_add_sync(0xffffffffu, a.cnt | (a.nx << 16));
         t.cnt = cx2 & 0xffffu;
         t.nx = cx2 >> 16;
@@ -486,6 +505,171 @@ __device__ __forceinline__ ViewTerms view_term(const Workspace &w, const SpShare
     t.Si = t.cnt > 0 ? sw * rcp_approx((float)t.cnt) : 0.f;                             // Eq. 9
     t.Vi = (t.cnt > 0 && t.nx > 0) ? t.Si * (sg * rcp_approx((float)t.nx)) : 0.f;       // Eq. 10
     t.Oi = (t.ny > 0 && (sh.term_mask & 4)) ? sh.eta * (1.f - S.minw) : 0.f;            // Eq. 11
+    return t;
+}
+
+// Neighbour views in which every pixel of the superpixel lands inside the
+// image, in front of both cameras, under hypothesis h (x: bit 4 k for view k),
+// or outside it (y).  Lane 4 k + c tests corner c of the offsets' box in view
+// k; inverse depth and homogeneous coordinate are affine in the offset, and a
+// homography takes a box in front of the camera into the hull of its corners,
+// so the corners decide for all pixels.  Margins: 0.1 px of the half pixel to
+// the window edge (a position's rounding is below 0.01 px up to 32767 px),
+// 1e-5 of the summed magnitudes for the sign of the inverse depth, a factor 4
+// for the range of the homogeneous coordinate.
+template <bool AFF>
+__device__ __forceinline__ uint2 views_inside(const SpShared &sh, const HypF &h, int nnb, float xy, int lane)
+{
+    const int k = lane >> 2;
+    bool in = false, front = false;
+    float x = 0.f, y = 0.f, xe = 0.f, ye = 0.f;
+    if (k < nnb) {
+        const SpView &sv = sh.view[k];
+        const float du = (lane & 1) ? sh.bx1 : sh.bx0, dv = (lane & 2) ? sh.by1 : sh.by0;
+        const float hw = fmaf(sv.qw, h.dgr, sv.hw_a);
+        const float Nw = AFF ? hw : fmaf(fmaf(sv.qw, h.g0, sv.P20), du, fmaf(fmaf(sv.qw, h.g1, sv.P21), dv, hw));
+        const float ex = fmaf(fmaf(sv.Dx, h.g0, sv.Pp00), du,
+                              fmaf(fmaf(sv.Dx, h.g1, sv.Pp01), dv, fmaf(sv.Dx, h.dgr, sv.Ex)));
+        const float ey = fmaf(fmaf(sv.Dy, h.g0, sv.Pp10), du,
+                              fmaf(fmaf(sv.Dy, h.g1, sv.Pp11), dv, fmaf(sv.Dy, h.dgr, sv.Ey)));
+        const float r = rcp_approx(Nw);
+        x = (float)(sv.xa_m + 0x4B400000) + ex * r;
+        y = (float)(sv.ya_m + 0x4B400000) + ey * r;
+        xe = (float)sv.Wi - 0.5f;
+        ye = (float)sv.Hi - 0.5f;
+        const float a = h.g0 * du, b = h.g1 * dv, gp = a + b + h.gr;
+        front = hw > 0.f && Nw > 0.25f * hw && Nw < 4.f * hw;
+        in = front && xy == 1.f && gp > 1e-5f * (fabsf(a) + fabsf(b) + fabsf(h.gr)) && x >= -0.4f && x <= xe - 0.1f &&
+             y >= -0.4f && y <= ye - 0.1f;
+    }
+    auto all4 = [](bool p) {
+        unsigned m = __ballot_sync(0xffffffffu, p);
+        m &= m >> 2;
+        return m & (m >> 1);
+    };
+    uint2 m;
+    m.x = all4(in);
+    m.y = all4(front && x < -0.6f) | all4(front && x > xe + 0.1f) | all4(front && y < -0.6f) |
+          all4(front && y > ye + 0.1f);
+    return m;
+}
+
+// view_term in a view of views_inside: no window, sign or slot tests, the
+// depth split without a factor (xy_eps = 0), the pixel count known.  Two slots
+// at a time in packed FP32, each operation rounded as the scalar one, the sums
+// in the same order: the same terms bit for bit.  With depth values NaN where
+// the map has none, val >= tw is X and val < tw is Y.
+//
+// 28 instructions per sample instead of 40 (affine pairs).  One rolled body
+// for most sizes: a body per slot count puts several on an SM at once where
+// label maps are uneven (perturbed grids, SLIC), and their instruction fetches
+// stall it (4 x 640x480, 12-pixel perturbed superpixels: 2.9 ms of propagation
+// with a body per slot count, 1.5 rolled).  Superpixels of 225 to 256 pixels,
+// the 16 x 16 cells of regular grids, keep an unrolled body of their own (16 x
+// 1080p: 62.8 ms rolled, 55.2 unrolled).  Bound now by the gathers' latency
+// (issue 65 % of the cycles, long scoreboard the largest stall).
+constexpr int INSIDE_SLOTS = 4;   // slots per iteration of the rolled body
+constexpr int UNROLLED_SLOTS = 8;
+
+// SL: 0 the rolled body, else an unrolled one for superpixels of SL slots
+template <int DOMAIN, bool AFF, int SL>
+__device__ __forceinline__ ViewTerms view_term_inside(const Workspace &w, const SpShared &sh, const HypF &h, int k,
+                                                      int lane, int count)
+{
+    const SpView &sv = sh.view[k];
+    const float hw = fmaf(sv.qw, h.dgr, sv.hw_a);
+    const float2 CX = dup2(fmaf(sv.Dx, h.dgr, sv.Ex)), CY = dup2(fmaf(sv.Dy, h.dgr, sv.Ey));
+    const float2 B0 = dup2(fmaf(sv.Dx, h.g0, sv.Pp00)), B1 = dup2(fmaf(sv.Dx, h.g1, sv.Pp01));
+    const float2 C0 = dup2(fmaf(sv.Dy, h.g0, sv.Pp10)), C1 = dup2(fmaf(sv.Dy, h.g1, sv.Pp11));
+    const float2 G0 = dup2(h.g0), G1 = dup2(h.g1), GR = dup2(h.gr), M = dup2(ROUND_MAGIC);
+    const float2 A20 = dup2(fmaf(sv.qw, h.g0, sv.P20)), A21 = dup2(fmaf(sv.qw, h.g1, sv.P21)), HW = dup2(hw);
+    const float cr = sh.S.cr, cg = sh.S.cg, cb = sh.S.cb;
+    const int Wi = sv.Wi, base = sv.ya_m * Wi + sv.xa_m;      // modulo 2^32
+    const float4 *map = sv.map;
+    const float2 Raff = dup2(AFF ? rcp_approx(hw) : 0.f);
+    float sw = 0.f, sg = 0.f;
+    unsigned nx = 0;
+    bool anyY = false;
+    auto tail = [&](bool act, float tx, float ty, float Nw, float gp, float val0) {
+        const int idx = __float_as_int(ty) * Wi + (__float_as_int(tx) + base);
+        const float4 c = __ldg(map + idx);
+        const float2 drg = fsub2(make_float2(c.x, c.y), make_float2(cr, cg));
+        const float2 d2 = fmul2(drg, drg);
+        const float db = c.z - cb;
+        const float om = ex2_approx(-fmaf(db, db, d2.x + d2.y));
+        const float val = DOMAIN == 0 ? val0 : Nw * rcp_approx(gp);
+        const float dd = val - c.w;
+        const float G = ex2_approx(-dd * dd);
+        const bool inX = act && (DOMAIN == 0 ? val >= c.w : val <= c.w);
+        const bool inY = act && (DOMAIN == 0 ? val < c.w : val > c.w);
+        if (act) sw += om;
+        if (inX) {
+            sg += G;
+            nx++;
+        }
+        anyY = anyY || inY;
+    };
+    auto pair = [&](int j, bool act0, bool act1) {            // slots j, j + 1
+        const float4 d = sh.px4[16 * j + lane];
+        const float2 du = make_float2(d.x, d.y), dv = make_float2(d.z, d.w);
+        const float2 gp = ffma2(G0, du, ffma2(G1, dv, GR));
+        const float2 ex = ffma2(B0, du, ffma2(B1, dv, CX)), ey = ffma2(C0, du, ffma2(C1, dv, CY));
+        float2 Nw = HW, R = Raff;
+        if (!AFF) {
+            Nw = ffma2(A20, du, ffma2(A21, dv, HW));
+            R = make_float2(rcp_approx(Nw.x), rcp_approx(Nw.y));
+        }
+        const float2 tx = ffma2(ex, R, M), ty = ffma2(ey, R, M), val = fmul2(gp, R);
+        tail(act0, tx.x, ty.x, Nw.x, gp.x, val.x);
+        tail(act1, tx.y, ty.y, Nw.y, gp.y, val.y);
+    };
+    if constexpr (SL > 0) {
+#pragma unroll
+        for (int j = 0; j < SL; j += 2)
+            pair(j, j + 1 < SL || lane + 32 * j < count, j + 1 < SL && (j + 2 < SL || lane + 32 * (j + 1) < count));
+    } else {
+        const int staged = min(count, 32 * SLOTS_MAX);
+        int j = 0;
+#pragma unroll 1
+        for (; 32 * (j + INSIDE_SLOTS) <= staged; j += INSIDE_SLOTS)
+#pragma unroll
+            for (int u = 0; u < INSIDE_SLOTS; u += 2) pair(j + u, true, true);
+#pragma unroll 1
+        for (; 32 * j < staged; j += 2) pair(j, lane + 32 * j < staged, lane + 32 * (j + 1) < staged);
+        // pixels beyond the staged slots, four steps of the warp at a time
+        auto listed = [&](int i) {
+            const unsigned pk = __ldg(w.sp_pix + sh.S.off + i);
+            const float du = (float)((int)(pk & 0xffff) - sh.S.ref.x), dv = (float)((int)(pk >> 16) - sh.S.ref.y);
+            const float gp = fmaf(h.g0, du, fmaf(h.g1, dv, h.gr));
+            const float Nw = AFF ? hw : fmaf(A20.x, du, fmaf(A21.x, dv, hw)), r = AFF ? Raff.x : rcp_approx(Nw);
+            tail(true, fmaf(fmaf(B0.x, du, fmaf(B1.x, dv, CX.x)), r, ROUND_MAGIC),
+                 fmaf(fmaf(C0.x, du, fmaf(C1.x, dv, CY.x)), r, ROUND_MAGIC), Nw, gp, gp * r);
+        };
+        int i = 32 * SLOTS_MAX;
+#pragma unroll 1
+        for (; i + 128 <= count; i += 128)
+#pragma unroll
+            for (int u = 0; u < 128; u += 32) listed(i + u + lane);
+#pragma unroll 1
+        for (i += lane; i < count; i += 32) listed(i);
+    }
+    __syncwarp();
+    ViewTerms t;
+    t.cnt = (unsigned)count;
+    t.nx = __reduce_add_sync(0xffffffffu, nx);
+    t.ny = __any_sync(0xffffffffu, anyY) ? 1u : 0u;
+    // both sums in one butterfly: after the exchange the lower half of the warp
+    // carries sw, the upper sg, each added in warp_sum's order
+    const bool up = lane >= 16;
+    float s2 = up ? sg : sw;
+    s2 += __shfl_xor_sync(0xffffffffu, up ? sw : sg, 16);
+#pragma unroll
+    for (int o = 8; o > 0; o >>= 1) s2 += __shfl_xor_sync(0xffffffffu, s2, o);
+    sw = __shfl_sync(0xffffffffu, s2, 0);
+    sg = __shfl_sync(0xffffffffu, s2, 16);
+    t.Si = sw * rcp_approx((float)t.cnt);
+    t.Vi = t.nx > 0 ? t.Si * (sg * rcp_approx((float)t.nx)) : 0.f;
+    t.Oi = (t.ny > 0 && (sh.term_mask & 4)) ? sh.eta * (1.f - sh.S.minw) : 0.f;
     return t;
 }
 
@@ -510,20 +694,26 @@ __device__ __forceinline__ float cand_bound(const SpShared &sh, float ec, float 
 // Energy of the candidate in batch slot `src` (x), summed over the views in
 // order; -1 as soon as its bound falls below Ebest (it can then neither beat
 // nor equal Ebest).  y: the views it was summed over.
-template <int DOMAIN, int SL, bool AFF, bool COOP>
+template <int DOMAIN, bool AFF, bool COOP>
 __device__ __noinline__ float2 eval_candidate(const Workspace &w, int src, float Ebest)
 {
     const int lane = threadIdx.x & 31;
     const SpShared &sh = sp_shared<COOP>();
-    const WarpSP S = sh.S;
+    const int nnb = sh.S.nnb, slots = slot_class(sh.S.n);
+    const int count = max(sh.S.n, 32 * (slots - 1));          // every slot but the last counts in full
     const HypF h = cand_load(g_cs[threadIdx.x >> 5], src);
+    const uint2 where = views_inside<AFF>(sh, h, nnb, DOMAIN == 0 ? sh.xy_lo : sh.xy_hi, lane);
     float ec = 0.f;
-    for (int k = 0; k < S.nnb; k++) {
-        const ViewTerms t = view_term<DOMAIN, SL, false, AFF>(w, sh, S, h, k, lane);
+    for (int k = 0; k < nnb; k++) {
+        ViewTerms t = {0.f, 0.f, 0.f, 0u, 0u, 0u};            // no pixel in view: no terms
+        if ((where.x >> (4 * k)) & 1u)
+            t = slots == UNROLLED_SLOTS ? view_term_inside<DOMAIN, AFF, UNROLLED_SLOTS>(w, sh, h, k, lane, count)
+                                        : view_term_inside<DOMAIN, AFF, 0>(w, sh, h, k, lane, count);
+        else if (!((where.y >> (4 * k)) & 1u)) t = view_term<DOMAIN, AFF>(w, sh, h, k, lane, slots, false);
         ec += t.Vi + t.Oi;
-        if (cand_bound(sh, ec, (float)(S.nnb - 1 - k), h.es) < Ebest) return make_float2(-1.f, (float)(k + 1));
+        if (cand_bound(sh, ec, (float)(nnb - 1 - k), h.es) < Ebest) return make_float2(-1.f, (float)(k + 1));
     }
-    return make_float2(cand_energy(sh, S.nnb, ec, h.es), (float)S.nnb);
+    return make_float2(cand_energy(sh, nnb, ec, h.es), (float)nnb);
 }
 
 // The best candidate of the batch `mask` in the warp's CandShared: the highest
@@ -539,7 +729,7 @@ __device__ __noinline__ float2 eval_candidate(const Workspace &w, int src, float
 // 69.5 ms; 8 x 1024x768 RGBA8, 6 iterations: 20.1 -> 13.5 ms.  Most of the
 // excluded candidates come from other surfaces: E_s rules them out before any
 // gather.
-template <int DOMAIN, int SL, bool AFF, bool COOP = false>
+template <int DOMAIN, bool AFF, bool COOP = false>
 __device__ __forceinline__ int best_of_batch(const Workspace &w, unsigned mask, float &Ebest, unsigned &views)
 {
     const int lane = threadIdx.x & 31;
@@ -553,7 +743,7 @@ __device__ __forceinline__ int best_of_batch(const Workspace &w, unsigned mask, 
         const int src = __ffs(__ballot_sync(0xffffffffu, ((mask >> lane) & 1u) && key == top)) - 1;
         if (__uint_as_float(top) < Ebest) break;
         mask &= ~(1u << src);
-        const float2 r = eval_candidate<DOMAIN, SL, AFF, COOP>(w, src, Ebest);
+        const float2 r = eval_candidate<DOMAIN, AFF, COOP>(w, src, Ebest);
         const float E = r.x;
         views += (unsigned)r.y;
         if (E > Ebest || (E == Ebest && best >= 0 && src < best)) {
@@ -695,7 +885,9 @@ __device__ bool setup_sp(const Workspace &w, const float4 *planes_in, int gs, in
         sh.view[lane] = sv;
     }
 
-    // pixel offsets of the first 32*SLOTS_MAX pixels (zero past the last pixel)
+    // pixel offsets of the first 32*SLOTS_MAX pixels (zero past the last pixel) and their box,
+    // which holds the anchor (the rounded centroid)
+    float x0 = 0.f, x1 = 0.f, y0 = 0.f, y1 = 0.f;
 #pragma unroll
     for (int jp = 0; jp < SLOTS_MAX / 2; jp++) {
         float4 d = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -711,8 +903,24 @@ __device__ bool setup_sp(const Workspace &w, const float4 *planes_in, int gs, in
             d.w = (float)((int)(pk >> 16) - S.ref.y);
         }
         sh.px4[32 * jp + lane] = d;
+        x0 = fminf(x0, fminf(d.x, d.y)); x1 = fmaxf(x1, fmaxf(d.x, d.y));
+        y0 = fminf(y0, fminf(d.z, d.w)); y1 = fmaxf(y1, fmaxf(d.z, d.w));
     }
-    if (lane == 0) sh.S = S;
+    for (int i = 32 * SLOTS_MAX + lane; i < S.n; i += 32) {   // pixels beyond the staged slots
+        const unsigned pk = __ldg(w.sp_pix + S.off + i);
+        const float du = (float)((int)(pk & 0xffff) - S.ref.x), dv = (float)((int)(pk >> 16) - S.ref.y);
+        x0 = fminf(x0, du); x1 = fmaxf(x1, du);
+        y0 = fminf(y0, dv); y1 = fmaxf(y1, dv);
+    }
+    __syncwarp();
+    // offsets are small integers: REDUX on them
+    const int ix0 = __reduce_min_sync(0xffffffffu, (int)x0), ix1 = __reduce_max_sync(0xffffffffu, (int)x1);
+    const int iy0 = __reduce_min_sync(0xffffffffu, (int)y0), iy1 = __reduce_max_sync(0xffffffffu, (int)y1);
+    if (lane == 0) {
+        sh.bx0 = (float)ix0; sh.bx1 = (float)ix1;
+        sh.by0 = (float)iy0; sh.by1 = (float)iy1;
+        sh.S = S;
+    }
     __syncwarp();
     return true;
 }
@@ -722,10 +930,10 @@ __device__ bool setup_sp(const Workspace &w, const float4 *planes_in, int gs, in
 // the camera; false for a missing vertex, a degenerate or a grazing
 // triangle.  The plane goes to slot `slot` of the warp's CandShared.
 template <int DOMAIN, bool COOP = false>
-__device__ __noinline__ bool triangle_candidate(const ViewDev &vd, double dnew, double ignew, int t, int slot)
+__device__ __noinline__ bool triangle_candidate(const ViewDev &vd, double dnew, double ignew, int t, CandShared &cs,
+                                                int slot)
 {
     const SpShared &sh = sp_shared<COOP>();
-    CandShared &cs = g_cs[threadIdx.x >> 5];
     const SpNb &A = sh.nb[t];
     const SpNb &B = sh.nb[(t + 1) & 7];
     if (!A.ok || !B.ok) return false;
@@ -755,10 +963,9 @@ __device__ __noinline__ bool triangle_candidate(const ViewDev &vd, double dnew, 
 // [d_min, d_max] or the plane is grazing.
 template <int DOMAIN, bool COOP = false>
 __device__ __noinline__ bool perturb_candidate(const ViewDev &vd, double dnew, double n0, double n1, double n2, int I,
-                                               int k, int slot)
+                                               int k, CandShared &cs, int slot)
 {
     const SpShared &sh = sp_shared<COOP>();
-    CandShared &cs = g_cs[threadIdx.x >> 5];
     const double rad = ldexp(vd.perturb_scale, 1 - I);
     double u[4];
     for (int j = 0; j < 4; j++) u[j] = perturb_u(vd.seed, vd.lf_index, vd.lv, sh.S.s, I, 4 * k + j);
@@ -780,20 +987,12 @@ __device__ __noinline__ bool perturb_candidate(const ViewDev &vd, double dnew, d
     return true;
 }
 
-// slots per lane for a superpixel of n pixels (the instantiated counts)
-__device__ __forceinline__ int slot_class(int n)
-{
-    const int s = (n + 31) >> 5;
-    return s <= 1 ? 1 : (s <= 8 ? s : SLOTS_MAX);
-}
-
 // ---------------------------------------------------------------------------
 // propagation + refinement
 // ---------------------------------------------------------------------------
 
-// one Jacobi update of superpixel gs by one warp (iteration `iter`, 1-based),
-// its pixels in SL slots per lane
-template <int DOMAIN, int SL, bool AFF>
+// one Jacobi update of superpixel gs by one warp (iteration `iter`, 1-based)
+template <int DOMAIN, bool AFF>
 __device__ __noinline__ void propagate_sp(const Workspace &w, int iter, int gs, const float4 *planes_in,
                                           float4 *planes_out, int *choice, float *energy, int batch)
 {
@@ -856,7 +1055,7 @@ __device__ __noinline__ void propagate_sp(const Workspace &w, int iter, int gs, 
         const unsigned mask = __ballot_sync(0xffffffffu, ok);
         n_hyp += __popc(mask);
         __syncwarp();
-        const int src = best_of_batch<DOMAIN, SL, AFF>(w, mask, Ebest, n_views);
+        const int src = best_of_batch<DOMAIN, AFF>(w, mask, Ebest, n_views);
         if (lane == 0 && base + src > 0 && src >= 0) {
             sh.best_m = base + src;
             sh.best_ig = cs.ig[src];
@@ -876,7 +1075,7 @@ __device__ __noinline__ void propagate_sp(const Workspace &w, int iter, int gs, 
     if (Ebest > -INFINITY && dnew > 0.0) {
         bool ok = false;
         if (lane < 8) {
-            ok = triangle_candidate<DOMAIN>(vd, dnew, ignew, lane, lane);
+            ok = triangle_candidate<DOMAIN>(vd, dnew, ignew, lane, cs, lane);
         } else if (lane < 8 + vd.perturb_k) {           // flagged variant: random planes around (dnew, n)
             double n0, n1, n2;
             if (best_m > 0) {
@@ -885,12 +1084,12 @@ __device__ __noinline__ void propagate_sp(const Workspace &w, int iter, int gs, 
                 const float4 cur = planes_in[gs];
                 n0 = cur.y; n1 = cur.z; n2 = cur.w;
             }
-            ok = perturb_candidate<DOMAIN>(vd, dnew, n0, n1, n2, ii, lane - 8, lane);
+            ok = perturb_candidate<DOMAIN>(vd, dnew, n0, n1, n2, ii, lane - 8, cs, lane);
         }
         const unsigned mask = __ballot_sync(0xffffffffu, ok);
         n_hyp += __popc(mask);
         __syncwarp();
-        best_t = best_of_batch<DOMAIN, SL, AFF>(w, mask, Ebest, n_views);
+        best_t = best_of_batch<DOMAIN, AFF>(w, mask, Ebest, n_views);
         if (lane == 0 && best_t >= 0) {
             sh.bnx = cs.nx[best_t];
             sh.bny = cs.ny[best_t];
@@ -911,9 +1110,7 @@ __device__ __noinline__ void propagate_sp(const Workspace &w, int iter, int gs, 
     }
 }
 
-// set-up and slot-count dispatch of one superpixel; each slot count is a
-// separate (not inlined) function, so that every variant gets its own
-// register allocation
+// set-up and update of one superpixel by one warp
 template <int DOMAIN, bool AFF>
 __device__ __forceinline__ void propagate_one(const Workspace &w, const Consts &c, int iter, int gs, int lane,
                                               const float4 *planes_in, float4 *planes_out, int *choice,
@@ -941,17 +1138,7 @@ __device__ __forceinline__ void propagate_one(const Workspace &w, const Consts &
         }
         return;
     }
-    switch (slot_class(S.n)) {
-    case 1: propagate_sp<DOMAIN, 1, AFF>(w, iter, gs, planes_in, planes_out, choice, energy, c.cand_batch); break;
-    case 2: propagate_sp<DOMAIN, 2, AFF>(w, iter, gs, planes_in, planes_out, choice, energy, c.cand_batch); break;
-    case 3: propagate_sp<DOMAIN, 3, AFF>(w, iter, gs, planes_in, planes_out, choice, energy, c.cand_batch); break;
-    case 4: propagate_sp<DOMAIN, 4, AFF>(w, iter, gs, planes_in, planes_out, choice, energy, c.cand_batch); break;
-    case 5: propagate_sp<DOMAIN, 5, AFF>(w, iter, gs, planes_in, planes_out, choice, energy, c.cand_batch); break;
-    case 6: propagate_sp<DOMAIN, 6, AFF>(w, iter, gs, planes_in, planes_out, choice, energy, c.cand_batch); break;
-    case 7: propagate_sp<DOMAIN, 7, AFF>(w, iter, gs, planes_in, planes_out, choice, energy, c.cand_batch); break;
-    case 8: propagate_sp<DOMAIN, 8, AFF>(w, iter, gs, planes_in, planes_out, choice, energy, c.cand_batch); break;
-    default: propagate_sp<DOMAIN, SLOTS_MAX, AFF>(w, iter, gs, planes_in, planes_out, choice, energy, c.cand_batch); break;
-    }
+    propagate_sp<DOMAIN, AFF>(w, iter, gs, planes_in, planes_out, choice, energy, c.cand_batch);
 }
 
 // ---------------------------------------------------------------------------
@@ -966,16 +1153,16 @@ __device__ __forceinline__ void propagate_one(const Workspace &w, const Consts &
 // lowest m on ties: the first maximum in m order, as the sequential scan
 // takes it).  The refinement candidates t go to warp t mod 4 the same way.
 // Every candidate's energy is computed by one warp with the code of the
-// per-warp form, so the results are the same bit for bit.  The point is
-// locality: the warps of a CTA reproject one superpixel into the same
-// neighbour view at the same time, so an SM's resident warps gather from 8
-// footprints instead of 32 and the candidates reuse them from L1.
-template <int DOMAIN, int SL, bool AFF>
+// per-warp form, so the results are the same bit for bit.  Which candidates
+// are summed in full depends on each warp's own best energy, not on timing.
+// The point is latency: a superpixel is done in a third to a half of the time,
+// which decides small inputs and the last wave of others (single_warp_count).
+template <int DOMAIN, bool AFF>
 __device__ __noinline__ void propagate_sp_coop(const Workspace &w, int iter, int gs, const float4 *planes_in,
                                                float4 *planes_out, int *choice, float *energy)
 {
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    SpShared &sh = g_shc[0];
+    SpShared &sh = g_sh[0];
     CandShared &cs = g_cs[wid];
     CoopShared &co = g_co;
     const WarpSP &S = sh.S;
@@ -1048,7 +1235,7 @@ __device__ __noinline__ void propagate_sp_coop(const Workspace &w, int iter, int
         const int nw = total > wid ? (total - wid + PROP_WARPS - 1) / PROP_WARPS : 0;
         const unsigned mask = nw >= 32 ? 0xffffffffu : ((1u << nw) - 1u);
         n_hyp += nw;
-        const int sbest = best_of_batch<DOMAIN, SL, AFF, true>(w, mask, Ebest, n_views);
+        const int sbest = best_of_batch<DOMAIN, AFF, true>(w, mask, Ebest, n_views);
         if (sbest >= 0 && lane == 0) {       // the round's winner of this warp: keep its plane
             co.E[wid] = Ebest;
             co.m[wid] = co.mi[wid][sbest];
@@ -1083,25 +1270,34 @@ __device__ __noinline__ void propagate_sp_coop(const Workspace &w, int iter, int
     const double dnew = best_m > 0 ? rcp64(best_ig) : (double)planes_in[gs].x;
     const double ignew = best_m > 0 ? best_ig : rcp64(dnew);
     if (Eprop > -INFINITY && dnew > 0.0) {
-        const int t = PROP_WARPS * lane + wid;
-        bool ok = false;
-        if (t < 8) {
-            ok = triangle_candidate<DOMAIN, true>(vd, dnew, ignew, t, lane);
-        } else if (t < 8 + vd.perturb_k) {   // flagged variant: random planes around (dnew, n)
-            double n0, n1, n2;
-            if (best_m > 0) {
-                n0 = pnx; n1 = pny; n2 = pnz;
-            } else {
-                const float4 cur = planes_in[gs];
-                n0 = cur.y; n1 = cur.z; n2 = cur.w;
+        // warp 0 builds the candidates, lane t candidate t, in the records of the
+        // warps that score them: FP64 for two lanes of every warp would occupy its
+        // narrow pipe four times as long
+        if (wid == 0) {
+            bool ok = false;
+            CandShared &dst = g_cs[lane & (PROP_WARPS - 1)];
+            if (lane < 8) {
+                ok = triangle_candidate<DOMAIN, true>(vd, dnew, ignew, lane, dst, lane / PROP_WARPS);
+            } else if (lane < 8 + vd.perturb_k) {   // flagged variant: random planes around (dnew, n)
+                double n0, n1, n2;
+                if (best_m > 0) {
+                    n0 = pnx; n1 = pny; n2 = pnz;
+                } else {
+                    const float4 cur = planes_in[gs];
+                    n0 = cur.y; n1 = cur.z; n2 = cur.w;
+                }
+                ok = perturb_candidate<DOMAIN, true>(vd, dnew, n0, n1, n2, ii, lane - 8, dst, lane / PROP_WARPS);
             }
-            ok = perturb_candidate<DOMAIN, true>(vd, dnew, n0, n1, n2, ii, t - 8, lane);
+            const unsigned okm = __ballot_sync(0xffffffffu, ok);
+            if (lane == 0) co.cnt[0] = (int)okm;
         }
-        const unsigned mask = __ballot_sync(0xffffffffu, ok);
+        __syncthreads();
+        const unsigned okm = (unsigned)co.cnt[0];
+        // bit s: candidate PROP_WARPS s + wid
+        const unsigned mask = __ballot_sync(0xffffffffu, lane < 32 / PROP_WARPS && ((okm >> (PROP_WARPS * lane + wid)) & 1u));
         n_hyp += __popc(mask);
-        __syncwarp();
         float Et = Eprop;                    // a winner has to beat the propagation's energy
-        const int st = best_of_batch<DOMAIN, SL, AFF, true>(w, mask, Et, n_views);
+        const int st = best_of_batch<DOMAIN, AFF, true>(w, mask, Et, n_views);
         if (lane == 0) {
             co.E[wid] = Et;
             co.m[wid] = st >= 0 ? PROP_WARPS * st + wid : -1;
@@ -1154,7 +1350,7 @@ __device__ __noinline__ void propagate_sp_coop(const Workspace &w, int iter, int
     }
 }
 
-// set-up (by warp 0) and slot-count dispatch of one superpixel for the CTA
+// set-up (by warp 0) and update of one superpixel by the CTA
 template <int DOMAIN, bool AFF>
 __device__ __forceinline__ void propagate_one_coop(const Workspace &w, const Consts &c, int iter, int gs,
                                                    const float4 *planes_in, float4 *planes_out, int *choice,
@@ -1172,7 +1368,7 @@ __device__ __forceinline__ void propagate_one_coop(const Workspace &w, const Con
             return;
         }
     }
-    SpShared &sh = g_shc[0];
+    SpShared &sh = g_sh[0];
     if (threadIdx.x < 32) {
         const dbl4 gc = w.sp_g[gs];
         WarpSP S;
@@ -1188,38 +1384,11 @@ __device__ __forceinline__ void propagate_one_coop(const Workspace &w, const Con
         }
         return;
     }
-    switch (slot_class(sh.S.n)) {
-    case 1: propagate_sp_coop<DOMAIN, 1, AFF>(w, iter, gs, planes_in, planes_out, choice, energy); break;
-    case 2: propagate_sp_coop<DOMAIN, 2, AFF>(w, iter, gs, planes_in, planes_out, choice, energy); break;
-    case 3: propagate_sp_coop<DOMAIN, 3, AFF>(w, iter, gs, planes_in, planes_out, choice, energy); break;
-    case 4: propagate_sp_coop<DOMAIN, 4, AFF>(w, iter, gs, planes_in, planes_out, choice, energy); break;
-    case 5: propagate_sp_coop<DOMAIN, 5, AFF>(w, iter, gs, planes_in, planes_out, choice, energy); break;
-    case 6: propagate_sp_coop<DOMAIN, 6, AFF>(w, iter, gs, planes_in, planes_out, choice, energy); break;
-    case 7: propagate_sp_coop<DOMAIN, 7, AFF>(w, iter, gs, planes_in, planes_out, choice, energy); break;
-    case 8: propagate_sp_coop<DOMAIN, 8, AFF>(w, iter, gs, planes_in, planes_out, choice, energy); break;
-    default: propagate_sp_coop<DOMAIN, SLOTS_MAX, AFF>(w, iter, gs, planes_in, planes_out, choice, energy); break;
-    }
+    propagate_sp_coop<DOMAIN, AFF>(w, iter, gs, planes_in, planes_out, choice, energy);
 }
 
-// persistent CTAs: one superpixel per CTA at a time, from the cost-ordered queue
-template <int DOMAIN, int MINB, bool AFF>
-__global__ void __launch_bounds__(32 * PROP_WARPS, MINB) k_propagate_coop(const __grid_constant__ Workspace w, Consts c,
-                                                                          int iter, const float4 *planes_in,
-                                                                          float4 *planes_out, int *choice,
-                                                                          float *energy)
-{
-    for (;;) {
-        if (threadIdx.x == 0) g_co.item = atomicAdd(&w.queue[1], 1);
-        __syncthreads();
-        const int item = g_co.item;
-        if (item >= w.S_total) break;
-        propagate_one_coop<DOMAIN, AFF>(w, c, iter, __ldg(w.order + item), planes_in, planes_out, choice, energy);
-        __syncthreads();                     // every thread is done with this superpixel's records
-    }
-}
-
-template <int DOMAIN, int MINB, bool AFF>
-__global__ void __launch_bounds__(32 * PROP_WARPS, MINB) k_propagate(const __grid_constant__ Workspace w, Consts c, int iter,
+template <int DOMAIN, bool AFF>
+__global__ void __launch_bounds__(32 * PROP_WARPS, PROP_CTAS) k_propagate(const __grid_constant__ Workspace w, Consts c, int iter,
                                                                      const float4 *planes_in, float4 *planes_out,
                                                                      int *choice, float *energy)
 {
@@ -1229,62 +1398,69 @@ __global__ void __launch_bounds__(32 * PROP_WARPS, MINB) k_propagate(const __gri
                                energy);
 }
 
-// persistent warps: superpixels taken from the cost-ordered queue, most expensive first
-template <int DOMAIN, int MINB, bool AFF>
-__global__ void __launch_bounds__(32 * PROP_WARPS, MINB) k_propagate_persistent(const __grid_constant__ Workspace w, Consts c, int iter,
-                                                                                const float4 *planes_in,
+// Persistent: superpixels taken from the cost-ordered queue, most expensive
+// first, the first `single` of them by single warps (queue[1]), the rest by
+// whole CTAs (queue[2]).
+template <int DOMAIN, bool AFF>
+__global__ void __launch_bounds__(32 * PROP_WARPS, PROP_CTAS) k_propagate_persistent(const __grid_constant__ Workspace w, Consts c, int iter,
+                                                                                int single, const float4 *planes_in,
                                                                                 float4 *planes_out, int *choice,
                                                                                 float *energy)
 {
     const int lane = threadIdx.x & 31;
-    for (;;) {
+    while (single > 0) {
         int item = 0;
         if (lane == 0) item = atomicAdd(&w.queue[1], 1);
         item = __shfl_sync(0xffffffffu, item, 0);
-        if (item >= w.S_total) break;
+        if (item >= single) break;
         propagate_one<DOMAIN, AFF>(w, c, iter, __ldg(w.order + item), lane, planes_in, planes_out, choice, energy);
         __syncwarp();
     }
+    if (single >= w.S_total) return;
+    for (;;) {
+        __syncthreads();                     // every thread is done with its superpixel's records
+        if (threadIdx.x == 0) g_co.item = single + atomicAdd(&w.queue[2], 1);
+        __syncthreads();
+        const int item = g_co.item;
+        if (item >= w.S_total) break;
+        propagate_one_coop<DOMAIN, AFF>(w, c, iter, __ldg(w.order + item), planes_in, planes_out, choice, energy);
+    }
 }
 
-template <int DOMAIN, int MINB, bool AFF>
+// Superpixels that single warps take when `slots` warps are resident: below a
+// few waves of them the last, partly filled wave decides the time, and its
+// superpixels go to whole CTAs unless they fill most of a wave.  A CTA costs
+// up to 1.3 times a warp's throughput per superpixel (set-up by one warp,
+// barriers) but takes a third to a half of its time: 900 superpixels 391 us in
+// single warps, 182 in CTAs; 2430 superpixels of 24 x 24 pixels 2994 and 1314;
+// 10800 (2.5 waves) 4200 in warps, 3296 with the half wave in CTAs; 18360 (4.3
+// waves) 4484 in warps, 5645 in CTAs.
+static int single_warp_count(int S, int slots)
+{
+    const int waves = S / slots, rest = S - waves * slots;
+    return waves >= 4 || 4 * rest >= 3 * slots ? S : waves * slots;
+}
+
+template <int DOMAIN, bool AFF>
 static cudaError_t launch_propagate_t(const Workspace &w, const Consts &c, const LaunchCfg &lc, int iter,
                                       const float4 *planes_in, float4 *planes_out, int *choice, float *energy,
                                       cudaStream_t st)
 {
-    if (lc.prop_persistent && lc.prop_coop) {
+    if (lc.prop_persistent) {
         int per_sm = 0;
         cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-            &per_sm, k_propagate_coop<DOMAIN, MINB, AFF>, 32 * PROP_WARPS, 0);
+            &per_sm, k_propagate_persistent<DOMAIN, AFF>, 32 * PROP_WARPS, 0);
         if (e != cudaSuccess) return e;
         const int grid = max(1, min(w.S_total, per_sm * lc.num_sms));
-        k_propagate_coop<DOMAIN, MINB, AFF><<<grid, 32 * PROP_WARPS, 0, st>>>(w, c, iter, planes_in, planes_out,
-                                                                              choice, energy);
-    } else if (lc.prop_persistent) {
-        int per_sm = 0;
-        cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-            &per_sm, k_propagate_persistent<DOMAIN, MINB, AFF>, 32 * PROP_WARPS, 0);
-        if (e != cudaSuccess) return e;
-        const int warps = (w.S_total + PROP_WARPS - 1) / PROP_WARPS;
-        const int grid = max(1, min(warps, per_sm * lc.num_sms));
-        k_propagate_persistent<DOMAIN, MINB, AFF><<<grid, 32 * PROP_WARPS, 0, st>>>(w, c, iter, planes_in,
+        const int single = lc.prop_coop ? 0 : single_warp_count(w.S_total, per_sm * lc.num_sms * PROP_WARPS);
+        k_propagate_persistent<DOMAIN, AFF><<<grid, 32 * PROP_WARPS, 0, st>>>(w, c, iter, single, planes_in,
                                                                                     planes_out, choice, energy);
     } else {
         const int blocks = (w.S_total + PROP_WARPS - 1) / PROP_WARPS;
-        k_propagate<DOMAIN, MINB, AFF><<<blocks, 32 * PROP_WARPS, 0, st>>>(w, c, iter, planes_in, planes_out, choice,
+        k_propagate<DOMAIN, AFF><<<blocks, 32 * PROP_WARPS, 0, st>>>(w, c, iter, planes_in, planes_out, choice,
                                                                            energy);
     }
     return cudaGetLastError();
-}
-
-template <int DOMAIN, int MINB>
-static cudaError_t launch_propagate_m(const Workspace &w, const Consts &c, const LaunchCfg &lc, int iter,
-                                      const float4 *planes_in, float4 *planes_out, int *choice, float *energy,
-                                      cudaStream_t st)
-{
-    return c.affine ? launch_propagate_t<DOMAIN, MINB, true>(w, c, lc, iter, planes_in, planes_out, choice, energy, st)
-                    : launch_propagate_t<DOMAIN, MINB, false>(w, c, lc, iter, planes_in, planes_out, choice, energy,
-                                                              st);
 }
 
 cudaError_t launch_propagate(const Workspace &w, const Consts &c0, const LaunchCfg &lc, int iter,
@@ -1293,12 +1469,11 @@ cudaError_t launch_propagate(const Workspace &w, const Consts &c0, const LaunchC
 {
     Consts c = c0;
     c.cand_batch = lc.prop_batch == 16 ? 16 : 32;
-    const bool eight = lc.prop_blocks >= 8;
     if (c.domain == 0)
-        return eight ? launch_propagate_m<0, 8>(w, c, lc, iter, planes_in, planes_out, choice, energy, st)
-                     : launch_propagate_m<0, 7>(w, c, lc, iter, planes_in, planes_out, choice, energy, st);
-    return eight ? launch_propagate_m<1, 8>(w, c, lc, iter, planes_in, planes_out, choice, energy, st)
-                 : launch_propagate_m<1, 7>(w, c, lc, iter, planes_in, planes_out, choice, energy, st);
+        return c.affine ? launch_propagate_t<0, true>(w, c, lc, iter, planes_in, planes_out, choice, energy, st)
+                        : launch_propagate_t<0, false>(w, c, lc, iter, planes_in, planes_out, choice, energy, st);
+    return c.affine ? launch_propagate_t<1, true>(w, c, lc, iter, planes_in, planes_out, choice, energy, st)
+                    : launch_propagate_t<1, false>(w, c, lc, iter, planes_in, planes_out, choice, energy, st);
 }
 
 // ---------------------------------------------------------------------------
@@ -1340,7 +1515,7 @@ __global__ void __launch_bounds__(128) k_score(const __grid_constant__ Workspace
     const HypF h = cand_load(cs, 0);
     float ec = 0.f;
     for (int k = 0; k < S.nnb; k++) {
-        const ViewTerms t = view_term<DOMAIN, SLOTS_MAX, true, false>(w, sh, S, h, k, lane);
+        const ViewTerms t = view_term<DOMAIN, false>(w, sh, h, k, lane, SLOTS_MAX, true);
         ec += t.Vi + t.Oi;
         if (lane == 0) {
             float *r = rec + LFD_TERMS_HEAD + k * LFD_TERMS_PER_VIEW;

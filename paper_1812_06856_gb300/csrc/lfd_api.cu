@@ -938,9 +938,8 @@ lfd_status enqueue_frame(lfd_ctx *ctx, const float *const *warm, float *const *c
 // Launch-shape autotuner: times each sweep and propagate variant on the bound
 // input (one warm-up run, then the median of three) and keeps the fastest.
 // Axes: sweep threads 128/256 x grid/persistent x row bands 1/16 of the
-// sweep's work order; propagation CTAs per SM 7/8 x grid/persistent
-// warps/cooperative CTAs x candidates per pass 16/32 x row bands 1/16
-// (timed on the first and the last iteration of the input).
+// sweep's work order; propagation grid/persistent warps/cooperative CTAs x
+// candidates per pass 16/32 x row bands 1/16 (timed on the first and the last iteration of the input).
 // Results do not depend on the shape (per-superpixel work is the same).
 lfd_status autotune(lfd_ctx *ctx, cudaStream_t st)
 {
@@ -999,40 +998,37 @@ lfd_status autotune(lfd_ctx *ctx, cudaStream_t st)
     if ((s = run_sweep(ctx, nullptr, st)) != LFD_OK) return s;
     if ((s = rasterize_state(ctx, ctx->d_planesA, nullptr, st)) != LFD_OK) return s;
     best_ms = 1e30f;
-    const int pb[2] = {7, 8}, cb[2] = {16, 32};
+    const int cb[2] = {16, 32};
     int it_last = 1;
     for (const LfInfo &l : ctx->lfs) it_last = std::max(it_last, l.p.iterations);
     for (int bi = 0; bi < 2; bi++) {
         if ((s = order(0, bands[bi])) != LFD_OK) return s;
         for (int pi = 0; pi < 3; pi++)        // grid, persistent warps, cooperative CTAs
-            for (int ki = 0; ki < 2; ki++)
-                for (int ci = 0; ci < 2; ci++) {
-                    ctx->lc.prop_blocks = pb[ki];
-                    ctx->lc.prop_persistent = pi > 0;
-                    ctx->lc.prop_coop = pi == 2;
-                    ctx->lc.prop_batch = cb[ci];
-                    float ms = 0;
-                    // the first and the last iteration: the candidate count falls with the
-                    // iteration index, and a shape can win on the first and lose on the rest
-                    auto fn = [&]() -> lfd_status {
-                        for (int it : {1, it_last}) {
-                            if (ctx->lc.prop_persistent) LFD_CUDA(cudaMemsetAsync(ctx->d_queue, 0, 4 * QUEUE_INTS, st));
-                            LFD_CUDA(launch_propagate(ctx->w, ctx->c, ctx->lc, it, ctx->d_planesA, ctx->d_planesB,
-                                                      nullptr, nullptr, st));
-                            if (it_last == 1) break;
-                        }
-                        return LFD_OK;
-                    };
-                    if ((s = time_it(fn, ms)) != LFD_OK) return s;
-                    if (ms < best_ms) {
-                        best_ms = ms;
-                        best.prop_blocks = pb[ki];
-                        best.prop_persistent = pi > 0;
-                        best.prop_coop = pi == 2;
-                        best.prop_batch = cb[ci];
-                        prop_bands = bands[bi];
+            for (int ci = 0; ci < 2; ci++) {
+                ctx->lc.prop_persistent = pi > 0;
+                ctx->lc.prop_coop = pi == 2;
+                ctx->lc.prop_batch = cb[ci];
+                float ms = 0;
+                // the first and the last iteration: the candidate count falls with the
+                // iteration index, and a shape can win on the first and lose on the rest
+                auto fn = [&]() -> lfd_status {
+                    for (int it : {1, it_last}) {
+                        if (ctx->lc.prop_persistent) LFD_CUDA(cudaMemsetAsync(ctx->d_queue, 0, 4 * QUEUE_INTS, st));
+                        LFD_CUDA(launch_propagate(ctx->w, ctx->c, ctx->lc, it, ctx->d_planesA, ctx->d_planesB,
+                                                  nullptr, nullptr, st));
+                        if (it_last == 1) break;
                     }
+                    return LFD_OK;
+                };
+                if ((s = time_it(fn, ms)) != LFD_OK) return s;
+                if (ms < best_ms) {
+                    best_ms = ms;
+                    best.prop_persistent = pi > 0;
+                    best.prop_coop = pi == 2;
+                    best.prop_batch = cb[ci];
+                    prop_bands = bands[bi];
                 }
+            }
     }
     // one band count serves both orders (enqueue_input builds both with it):
     // the propagation's choice, the larger share of a frame's time

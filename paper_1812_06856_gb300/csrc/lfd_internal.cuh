@@ -8,7 +8,7 @@
 //   sp_cnt, sp_ref (rounded centroid), sp_cen (FP64 centroid), sp_col {r,g,b,minw}
 //   quad textures                per pixel the 2x2 block (x,y),(x+1,y),(x,y+1),(x+1,y+1),
 //                                edges clamped: one load serves a bilinear sample
-//   maps                         per pixel float4 {superpixel mean colour, depth value},
+//   maps                         per pixel float4 {superpixel mean colour, depth value (NaN: none)},
 //                                written by the rasteriser, gathered by the energy kernel
 //   sp_g / sp_rc                 per-superpixel plane coefficients of the current state
 #pragma once
@@ -254,21 +254,19 @@ __device__ __forceinline__ void ring_dir(int d, int &dx, int &dy)
 struct LaunchCfg {
     int sweep_threads;       // 128 or 256 threads (labels) per CTA
     int sweep_persistent;    // 1: persistent CTAs over a cost-ordered queue
-    int prop_blocks;         // 7 or 8 resident 4-warp CTAs per SM (register budget)
+    int prop_blocks;         // 7 or 8, as given (one register budget: PROP_CTAS)
     int prop_persistent;     // 1: persistent warps over a cost-ordered queue
     int num_sms;
     int prop_batch;          // 16 or 32 candidate planes per pass over the neighbour views
     int order_bands;         // 1 or 16 row bands in the work orders
-    int prop_coop;           // 1: persistent CTAs whose 4 warps share one superpixel (k_propagate_coop)
+    int prop_coop;           // 1: persistent CTAs whose 4 warps share one superpixel (propagate_sp_coop)
 };
 
-cudaError_t launch_sp_count(const Workspace &w, int V, int max_px, int *cnt, int4 *bbox, cudaStream_t st);
 cudaError_t launch_sp_scan(const Workspace &w, int V, const int *cnt, int *off, cudaStream_t st);
 cudaError_t launch_sp_collect(const Workspace &w, const Consts &c, const int4 *bbox, const int *cnt, unsigned *pix,
                               double2 *cen, int2 *ref, float4 *col, cudaStream_t st);
 cudaError_t launch_sp_minw(const Workspace &w, const Consts &c, float4 *col, cudaStream_t st);
 cudaError_t launch_quads(const Workspace &w, int V, int max_px, int fmt, cudaStream_t st);
-// mode 0: pixel-slot classes ceil(n/32) (propagation); mode 1: power-of-two classes floor(log2 n) (sweep)
 // keys of the work orders' counting sort: 17 size classes x 16 row bands
 constexpr int ORDER_CLASSES = 17;
 constexpr int ORDER_BANDS = 16;
@@ -289,12 +287,6 @@ inline int label_class(int L)
         if (L <= LCLASS_THREADS[c]) return c;
     return LCLASSES - 1;
 }
-// mode 0: propagation order (pixel-slot class, band); 1: sweep order
-// (power-of-two size class, band); 2: stable partition of `in` by the
-// label-count class of each superpixel's light field.  bands: 1 ..
-// ORDER_BANDS row bands inside a size class.  in: NULL = index order.
-cudaError_t launch_sp_order(const Workspace &w, int *order, int *hist, int mode, int bands, const int *in,
-                            cudaStream_t st);  // hist: ORDER_KEYS ints
 // sweep of the superpixels order_sweep[base .. base + count) with CTAs of
 // `threads` threads (one of LCLASS_THREADS), queue counter queue[qidx]
 cudaError_t launch_sweep(const Workspace &w, const Consts &c, const LaunchCfg &lc, int threads, int base, int count,
@@ -305,7 +297,6 @@ cudaError_t launch_rasterize(const Workspace &w, const Consts &c, float *const *
 cudaError_t launch_propagate(const Workspace &w, const Consts &c, const LaunchCfg &lc, int iter,
                              const float4 *planes_in, float4 *planes_out, int *choice, float *energy,
                              cudaStream_t st);
-cudaError_t launch_fuse(const FuseArgs &a, long long zbuf_words, int max_px, cudaStream_t st);
 cudaError_t launch_score(const Workspace &w, const Consts &c, const float4 *planes_state, int nq, const lfd_query *q,
                          float *out, cudaStream_t st);
 }  // namespace lfd
