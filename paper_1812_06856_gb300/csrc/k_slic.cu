@@ -59,8 +59,8 @@ __device__ __forceinline__ int cell_edge(int k, int size, int n)
 }
 
 // The scratch is cell-major: cell c = cy GW + cx holds its pixels, row by row,
-// at entries c stride .. of `lab` and `code`, so that a warp reads a cell, or
-// the three cells of a window's row, as one contiguous run.  A Lab entry's
+// at entries c stride .. of `lab`, so that a warp reads
+// it as one contiguous run.  A Lab entry's
 // fourth word is (y << 16 | x).  The entries past a cell's last pixel hold a
 // NaN colour and a negative fourth word: they pick no centre.
 //
@@ -134,179 +134,195 @@ __device__ __forceinline__ int slic_fix(float v)
 }
 
 // A cell's pixels pick the nearest of the 3x3 cells' centres (ties to the
-// first in row-major order): code 0..8, or 255 when every distance is NaN (a
-// colour that is not finite keeps its own cell and enters no mean).  FINAL
-// writes the labels instead.  Lanes take pixels in pairs: a centre's
-// shared-memory broadcast, every component twice, feeds the packed FP32
-// operations for both; each operation rounds as the scalar one.
+// first in row-major order; the own cell, and no mean, when every distance is
+// NaN).  FINAL writes the labels; otherwise the picks go into the sums {L, a, b
+// in fixed point, x, y, count} of the cell's pixels per centre picked,
+// s.sums[cell][9][6], which k_slic_update adds up centre by centre: no atomics.
+//
+// Lanes take pixels in pairs: a centre's shared-memory broadcast, every
+// component twice, feeds the packed FP32 operations for both; each operation
+// rounds as the scalar one.  After 128 pixels (four a lane) the warp sums the
+// picks of one centre after the other, of those present: lane sums fit 32 bits
+// (four values below 2^26), a REDUX each for their low and high halves, and
+// lane j keeps centre j's totals.  Offsets in the cell are summed as one word
+// (dy << 16 | dx) unless WIDE (cells above 256 pixels across).
 //
 // 8 x 1024x768 RGBA8, 4015 cells of 14 x 14 pixels per view, 10 iterations:
-// 46 us an assignment and 80 us an update, 1.44 ms in all; one CTA per cell
-// that also added every pixel to its winner's sums (REDUX per quantity and
-// winner, 64-bit atomics) took 272 us an iteration, 3.02 ms in all.  Both
-// kernels are bound by issue and latency together (63 % issue-active at 40
-// warps per SM); the Lab entries (108 MB) come from HBM once per iteration,
-// 2.2 TB/s.
-template <bool FINAL>
-__global__ void __launch_bounds__(32 * SLIC_WARPS, 5) k_slic_assign(const __grid_constant__ SlicBatch b, int parity,
-                                                                 int wpc)
+// 103 us an assignment with its sums, 8 us an update, 1.30 ms in all; with one
+// byte per pixel out and the sums gathered by a warp per centre from its 3x3
+// cells 46 and 80 us, 1.43 ms; with one CTA per cell, REDUX per quantity and
+// winner and 64-bit atomics 272 us an iteration, 3.02 ms.  Bound by issue; 3
+// CTAs per SM at 80 registers (4 at 64 spill: 1.34 ms).
+template <bool FINAL, bool WIDE>
+__global__ void __launch_bounds__(32 * SLIC_WARPS, 3) k_slic_assign(const __grid_constant__ SlicBatch b, int parity,
+                                                                    int wpc)
 {
     const SlicView &s = b.v[blockIdx.y];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const int c = blockIdx.x * (SLIC_WARPS / wpc) + wid / wpc;
-    if (c >= s.GW * s.GH) return;                // whole warp
-    const float *centres = parity ? s.centres2 : s.centres;
-    const float2 wxy = dup2(b.wxy[blockIdx.y]);
     __shared__ float4 cen[SLIC_WARPS][9][3];     // {L, L, a, a}, {b, b, x, x}, {y, y, -, -}
-    const int cx = c % s.GW, cy = c / s.GW;
-    if (lane < 9) {
-        const int nx = cx + lane % 3 - 1, ny = cy + lane / 3 - 1;
-        const bool in = nx >= 0 && ny >= 0 && nx < s.GW && ny < s.GH;
-        const float *o = centres + 5 * (long long)(in ? ny * s.GW + nx : c);
-        const float L = in ? o[0] : INFINITY;    // no cell there: an infinite distance wins nothing
-        cen[wid][lane][0] = make_float4(L, L, o[1], o[1]);
-        cen[wid][lane][1] = make_float4(o[2], o[2], o[3], o[3]);
-        cen[wid][lane][2] = make_float4(o[4], o[4], 0.f, 0.f);
-    }
-    __syncwarp();
-    const float4 *lab = s.lab + (long long)c * s.stride;
-    unsigned char *code = s.code + (long long)c * s.stride;
-    for (int i0 = (wid % wpc) * 64 + lane; i0 - lane < s.stride; i0 += 64 * wpc) {
-        const int i1 = i0 + 32;
-        const float4 l0 = __ldg(lab + min(i0, s.stride - 1)), l1 = __ldg(lab + min(i1, s.stride - 1));
-        const int p0 = __float_as_int(l0.w), p1 = __float_as_int(l1.w);
-        const float2 vl = make_float2(l0.x, l1.x), va = make_float2(l0.y, l1.y), vb = make_float2(l0.z, l1.z);
-        const float2 vx = make_float2((float)(p0 & 0xffff), (float)(p1 & 0xffff));
-        const float2 vy = make_float2((float)(p0 >> 16), (float)(p1 >> 16));
-        float best0 = INFINITY, best1 = INFINITY;
-        int k0 = 255, k1 = 255;
-#pragma unroll
-        for (int j = 0; j < 9; j++) {
-            const float4 q0 = cen[wid][j][0], q1 = cen[wid][j][1];
-            const float2 q2 = *(const float2 *)&cen[wid][j][2];
-            const float2 dl = fsub2(vl, make_float2(q0.x, q0.y)), da = fsub2(va, make_float2(q0.z, q0.w));
-            const float2 db = fsub2(vb, make_float2(q1.x, q1.y)), dx = fsub2(vx, make_float2(q1.z, q1.w));
-            const float2 dy = fsub2(vy, q2);
-            const float2 col = ffma2(dl, dl, ffma2(da, da, fmul2(db, db)));
-            const float2 D = ffma2(wxy, ffma2(dx, dx, fmul2(dy, dy)), col);
-            if (D.x < best0) { best0 = D.x; k0 = j; }
-            if (D.y < best1) { best1 = D.y; k1 = j; }
-        }
-        if (FINAL) {
-            const int j0 = k0 == 255 ? 4 : k0, j1 = k1 == 255 ? 4 : k1;
-            if (i0 < s.stride && p0 >= 0)
-                s.labels[(long long)(p0 >> 16) * s.W + (p0 & 0xffff)] = c + (j0 / 3 - 1) * s.GW + j0 % 3 - 1;
-            if (i1 < s.stride && p1 >= 0)
-                s.labels[(long long)(p1 >> 16) * s.W + (p1 & 0xffff)] = c + (j1 / 3 - 1) * s.GW + j1 % 3 - 1;
-        } else {
-            if (i0 < s.stride) code[i0] = (unsigned char)k0;
-            if (i1 < s.stride) code[i1] = (unsigned char)k1;
-        }
-    }
-}
-
-// exact sum over the warp of 64-bit values below 2^62 in magnitude: three
-// 22-bit limbs, one REDUX each (the top one signed)
-__device__ __forceinline__ long long warp_sum64(long long v)
-{
-    const unsigned lo = __reduce_add_sync(0xffffffffu, (unsigned)v & 0x3fffffu);
-    const unsigned mid = __reduce_add_sync(0xffffffffu, (unsigned)(v >> 22) & 0x3fffffu);
-    const int hi = __reduce_add_sync(0xffffffffu, (int)(v >> 44));
-    return ((long long)hi << 44) + ((long long)mid << 22) + (long long)lo;
-}
-
-// A centre becomes the mean of the pixels that picked it (kept when there are
-// none): its warps find them among the codes of the centre's 3x3 cells, four a
-// word and a window row (three cells) as one run, list them in shared memory
-// and sum them with full lanes, {L, a, b} in fixed point.
-constexpr int SLIC_LIST = 512;
-
-__global__ void __launch_bounds__(32 * SLIC_WARPS, 5) k_slic_update(const __grid_constant__ SlicBatch b, int parity,
-                                                                 int wpc)
-{
-    const SlicView &s = b.v[blockIdx.y];
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    const int c = blockIdx.x * (SLIC_WARPS / wpc) + wid / wpc;
-    __shared__ int list[SLIC_WARPS][SLIC_LIST];
-    __shared__ long long tot[SLIC_WARPS][6];
+    __shared__ long long part[FINAL ? 1 : SLIC_WARPS][9][6];
     const bool here = c < s.GW * s.GH;           // whole warp
-    long long sum[6] = {0, 0, 0, 0, 0, 0};       // L, a, b (fixed point), x, y, count
+    long long tot[6] = {0, 0, 0, 0, 0, 0};       // lane j: centre j's sums
     if (here) {
+        const float *centres = parity ? s.centres2 : s.centres;
+        const float2 wxy = dup2(b.wxy[blockIdx.y]);
         const int cx = c % s.GW, cy = c / s.GW;
-        const unsigned lt = (1u << lane) - 1u;
-        const int words = s.stride >> 2;
-        int have = 0;
-        auto drain = [&]() {                     // at most 16 entries a lane: 32-bit sums
-            __syncwarp();
-            int q[6] = {0, 0, 0, 0, 0, 0};
-#pragma unroll 4
-            for (int e = lane; e < have; e += 32) {
-                const float4 l = __ldg(s.lab + list[wid][e]);
-                const int p = __float_as_int(l.w);
-                q[0] += slic_fix(l.x);
-                q[1] += slic_fix(l.y);
-                q[2] += slic_fix(l.z);
-                q[3] += p & 0xffff;
-                q[4] += p >> 16;
-                q[5]++;
+        const int x0 = cell_edge(cx, s.W, s.GW), y0 = cell_edge(cy, s.H, s.GH);
+        if (lane < 9) {
+            const int nx = cx + lane % 3 - 1, ny = cy + lane / 3 - 1;
+            const bool in = nx >= 0 && ny >= 0 && nx < s.GW && ny < s.GH;
+            const float *o = centres + 5 * (long long)(in ? ny * s.GW + nx : c);
+            const float L = in ? o[0] : INFINITY;    // no cell there: an infinite distance wins nothing
+            cen[wid][lane][0] = make_float4(L, L, o[1], o[1]);
+            cen[wid][lane][1] = make_float4(o[2], o[2], o[3], o[3]);
+            cen[wid][lane][2] = make_float4(o[4], o[4], 0.f, 0.f);
+        }
+        __syncwarp();
+        const float4 *lab = s.lab + (long long)c * s.stride;
+#pragma unroll 1
+        for (int base = (wid % wpc) * 128; base < s.stride; base += 128 * wpc) {
+            float4 px[4];
+            int pick[4];
+#pragma unroll
+            for (int u = 0; u < 4; u++) px[u] = __ldg(lab + min(base + 32 * u + lane, s.stride - 1));
+            float2 vl[2], va[2], vb[2], vx[2], vy[2], best[2];
+#pragma unroll
+            for (int h = 0; h < 2; h++) {
+                const float4 l0 = px[2 * h], l1 = px[2 * h + 1];
+                const int p0 = __float_as_int(l0.w), p1 = __float_as_int(l1.w);
+                vl[h] = make_float2(l0.x, l1.x);
+                va[h] = make_float2(l0.y, l1.y);
+                vb[h] = make_float2(l0.z, l1.z);
+                vx[h] = make_float2((float)(p0 & 0xffff), (float)(p1 & 0xffff));
+                vy[h] = make_float2((float)(p0 >> 16), (float)(p1 >> 16));
+                best[h] = make_float2(INFINITY, INFINITY);
+                pick[2 * h] = pick[2 * h + 1] = 255;
             }
 #pragma unroll
-            for (int k = 0; k < 6; k++) sum[k] += q[k];
-            have = 0;
-            __syncwarp();
-        };
-        const int xl = max(cx - 1, 0), cells = min(cx + 1, s.GW - 1) - xl + 1;   // of a window row
-        const int run = cells * words;
-        for (int ny = max(cy - 1, 0); ny <= min(cy + 1, s.GH - 1); ny++) {
-            const int first = (ny * s.GW + xl) * s.stride;
-            const unsigned *code = (const unsigned *)(s.code + first);
-            // this centre as the row's first cell numbers it; one less per cell to the right
-            const int want = (cy - ny + 1) * 3 + (cx - xl + 1);
-#pragma unroll 2
-            for (int w0 = (wid % wpc) * 32; w0 < run; w0 += 32 * wpc) {
-                const int wi = w0 + lane;
-                const int at = want - (wi >= words ? 1 : 0) - (wi >= 2 * words ? 1 : 0);
-                const unsigned m = wi < run ? __vcmpeq4(__ldg(code + min(wi, run - 1)), (unsigned)at * 0x01010101u) : 0u;
-                if (have + 128 > SLIC_LIST) drain();
+            for (int j = 0; j < 9; j++) {
+                const float4 q0 = cen[wid][j][0], q1 = cen[wid][j][1];
+                const float2 q2 = *(const float2 *)&cen[wid][j][2];
 #pragma unroll
-                for (int y = 0; y < 4; y++) {
-                    const bool hit = (m >> (8 * y)) & 1u;
-                    const unsigned bal = __ballot_sync(0xffffffffu, hit);
-                    if (hit) list[wid][have + __popc(bal & lt)] = first + 4 * wi + y;
-                    have += __popc(bal);
+                for (int h = 0; h < 2; h++) {
+                    const float2 dl = fsub2(vl[h], make_float2(q0.x, q0.y)), da = fsub2(va[h], make_float2(q0.z, q0.w));
+                    const float2 db = fsub2(vb[h], make_float2(q1.x, q1.y)), dx = fsub2(vx[h], make_float2(q1.z, q1.w));
+                    const float2 dy = fsub2(vy[h], q2);
+                    const float2 col = ffma2(dl, dl, ffma2(da, da, fmul2(db, db)));
+                    const float2 D = ffma2(wxy, ffma2(dx, dx, fmul2(dy, dy)), col);
+                    if (D.x < best[h].x) { best[h].x = D.x; pick[2 * h] = j; }
+                    if (D.y < best[h].y) { best[h].y = D.y; pick[2 * h + 1] = j; }
                 }
             }
-        }
-        drain();
+            // past the cell's entries (the clamped loads): no pick
 #pragma unroll
-        for (int q = 0; q < 6; q++) sum[q] = warp_sum64(sum[q]);
-    }
-    if (lane < 6) {
-        long long v = 0;
+            for (int u = 0; u < 4; u++)
+                if (base + 32 * u + lane >= s.stride) pick[u] = 256;
+            if (FINAL) {
 #pragma unroll
-        for (int q = 0; q < 6; q++) v = lane == q ? sum[q] : v;
-        tot[wid][lane] = v;
+                for (int u = 0; u < 4; u++) {
+                    const int p = __float_as_int(px[u].w), j = pick[u] == 255 ? 4 : pick[u];
+                    if (pick[u] < 256 && p >= 0)
+                        s.labels[(long long)(p >> 16) * s.W + (p & 0xffff)] = c + (j / 3 - 1) * s.GW + j % 3 - 1;
+                }
+                continue;
+            }
+            int q[4][3], off[4];
+            unsigned mine = 0;
+#pragma unroll
+            for (int u = 0; u < 4; u++) {
+                const int p = __float_as_int(px[u].w);
+                q[u][0] = slic_fix(px[u].x);
+                q[u][1] = slic_fix(px[u].y);
+                q[u][2] = slic_fix(px[u].z);
+                off[u] = (((p >> 16) - y0) << 16) | ((p & 0xffff) - x0);
+                mine |= pick[u] < 9 ? 1u << pick[u] : 0u;
+            }
+            unsigned present = __reduce_or_sync(0xffffffffu, mine);
+            while (present) {
+                const int j = __ffs(present) - 1;
+                present &= present - 1;
+                int t[3] = {0, 0, 0}, xy = 0, yy = 0, n = 0;
+#pragma unroll
+                for (int u = 0; u < 4; u++)
+                    if (pick[u] == j) {
+                        t[0] += q[u][0];
+                        t[1] += q[u][1];
+                        t[2] += q[u][2];
+                        if (WIDE) {
+                            xy += off[u] & 0xffff;
+                            yy += off[u] >> 16;
+                        } else {
+                            xy += off[u];
+                        }
+                        n++;
+                    }
+                long long r[6];
+#pragma unroll
+                for (int k = 0; k < 3; k++) {
+                    const unsigned lo = __reduce_add_sync(0xffffffffu, (unsigned)t[k] & 0xffffu);
+                    const int hi = __reduce_add_sync(0xffffffffu, t[k] >> 16);
+                    r[k] = ((long long)hi << 16) + lo;
+                }
+                const unsigned sxy = __reduce_add_sync(0xffffffffu, (unsigned)xy);
+                const unsigned sn = __reduce_add_sync(0xffffffffu, (unsigned)n);
+                const unsigned sy = WIDE ? __reduce_add_sync(0xffffffffu, (unsigned)yy) : sxy >> 16;
+                r[3] = (long long)(WIDE ? sxy : sxy & 0xffffu) + (long long)sn * x0;
+                r[4] = (long long)sy + (long long)sn * y0;
+                r[5] = sn;
+                if (lane == j)
+#pragma unroll
+                    for (int k = 0; k < 6; k++) tot[k] += r[k];
+            }
+        }
     }
-    __syncthreads();
-    // the means, one lane per centre of the CTA: FP64 is taken once for all of
-    // them (its pipe is 16 times narrower than FP32's)
-    const int per = SLIC_WARPS / wpc, cl = blockIdx.x * per + lane;
-    if (wid == 0 && lane < per && cl < s.GW * s.GH) {
-        long long t[6];
-        for (int q = 0; q < 6; q++) {
-            t[q] = 0;
-            for (int k = 0; k < wpc; k++) t[q] += tot[lane * wpc + k][q];
-        }
-        const float *cin = (parity ? s.centres2 : s.centres) + 5 * (long long)cl;
-        float *o = (parity ? s.centres : s.centres2) + 5 * (long long)cl;
-        if (t[5] > 0) {
-            const double r = 1.0 / (double)t[5];
-            for (int j = 0; j < 3; j++) o[j] = (float)((double)t[j] * r * (1.0 / SLIC_FIX));
-            o[3] = (float)((double)t[3] * r);
-            o[4] = (float)((double)t[4] * r);
-        } else {
-            for (int j = 0; j < 5; j++) o[j] = cin[j];
-        }
+    if (FINAL) return;
+    if (wpc > 1) {                               // the warps that share the cell
+        if (lane < 9)
+#pragma unroll
+            for (int k = 0; k < 6; k++) part[wid][lane][k] = tot[k];
+        __syncthreads();
+        if (wid % wpc) return;
+        if (lane < 9)
+            for (int o = 1; o < wpc; o++)
+#pragma unroll
+                for (int k = 0; k < 6; k++) tot[k] += part[wid + o][lane][k];
+    }
+    if (here && lane < 9) {
+        longlong2 *out = (longlong2 *)(s.sums + 54 * (long long)c + 6 * lane);
+        out[0] = make_longlong2(tot[0], tot[1]);
+        out[1] = make_longlong2(tot[2], tot[3]);
+        out[2] = make_longlong2(tot[4], tot[5]);
+    }
+}
+
+// a centre becomes the mean of the pixels that picked it in its 3x3 cells
+// (kept when there are none)
+__global__ void __launch_bounds__(128) k_slic_update(const __grid_constant__ SlicBatch b, int parity)
+{
+    const SlicView &s = b.v[blockIdx.y];
+    const int c = blockIdx.x * 128 + threadIdx.x;
+    if (c >= s.GW * s.GH) return;
+    const int cx = c % s.GW, cy = c / s.GW;
+    long long t[6] = {0, 0, 0, 0, 0, 0};
+#pragma unroll
+    for (int q = 0; q < 9; q++) {
+        const int nx = cx + q % 3 - 1, ny = cy + q / 3 - 1;
+        if (nx < 0 || ny < 0 || nx >= s.GW || ny >= s.GH) continue;
+        // this centre as that cell numbers it
+        const longlong2 *in = (const longlong2 *)(s.sums + 54 * (long long)(ny * s.GW + nx) + 6 * (8 - q));
+        const longlong2 u = __ldg(in), v = __ldg(in + 1), w = __ldg(in + 2);
+        t[0] += u.x; t[1] += u.y; t[2] += v.x; t[3] += v.y; t[4] += w.x; t[5] += w.y;
+    }
+    const float *cin = (parity ? s.centres2 : s.centres) + 5 * (long long)c;
+    float *o = (parity ? s.centres : s.centres2) + 5 * (long long)c;
+    if (t[5] > 0) {
+        const double r = 1.0 / (double)t[5];
+        for (int j = 0; j < 3; j++) o[j] = (float)((double)t[j] * r * (1.0 / SLIC_FIX));
+        o[3] = (float)((double)t[3] * r);
+        o[4] = (float)((double)t[4] * r);
+    } else {
+        for (int j = 0; j < 5; j++) o[j] = cin[j];
     }
 }
 
@@ -314,14 +330,18 @@ cudaError_t launch_slic(const SlicBatch &b, const float *const *centres_in, int 
                         float *const *centres_out, cudaStream_t st)
 {
     // warps per cell: one as long as that fills the chip (152 SMs, 32 warps
-    // each), more for few or large cells while each warp keeps a step of 64 pixels
+    // each), more for few or large cells while each warp keeps a step of 128 pixels
     int wpc = 1;
-    while (wpc < SLIC_WARPS && b.max_stride > 64 * wpc &&
+    while (wpc < SLIC_WARPS && b.max_stride > 128 * wpc &&
            (b.max_stride > 1024 * wpc || (long long)b.max_cells * b.n * wpc < 152 * 32))
         wpc *= 2;
     const int per_cta = SLIC_WARPS / wpc;
     const dim3 grid((b.max_cells + per_cta - 1) / per_cta, b.n);
     constexpr int threads = 32 * SLIC_WARPS;
+    const dim3 g_cells((b.max_cells + 127) / 128, b.n);
+    bool wide = false;                       // (dy << 16 | dx) sums of 128 pixels fit below 256 x 256
+    for (int v = 0; v < b.n; v++)
+        wide = wide || b.v[v].W > 256 * b.v[v].GW || b.v[v].H > 256 * b.v[v].GH;
     k_slic_lab<<<grid, threads, 0, st>>>(b, wpc);
     bool seeds = false;
     for (int v = 0; v < b.n; v++) {
@@ -344,11 +364,12 @@ cudaError_t launch_slic(const SlicBatch &b, const float *const *centres_in, int 
         k_slic_seeds<<<dim3((b.max_cells + 127) / 128, k), 128, 0, st>>>(bs);
     }
     for (int it = 0; it < iterations; it++) {
-        k_slic_assign<false><<<grid, threads, 0, st>>>(b, it & 1, wpc);
-        k_slic_update<<<grid, threads, 0, st>>>(b, it & 1, wpc);
+        if (wide) k_slic_assign<false, true><<<grid, threads, 0, st>>>(b, it & 1, wpc);
+        else k_slic_assign<false, false><<<grid, threads, 0, st>>>(b, it & 1, wpc);
+        k_slic_update<<<g_cells, 128, 0, st>>>(b, it & 1);
     }
     const int parity = iterations & 1;
-    k_slic_assign<true><<<grid, threads, 0, st>>>(b, parity, wpc);
+    k_slic_assign<true, false><<<grid, threads, 0, st>>>(b, parity, wpc);
     for (int v = 0; v < b.n && centres_out; v++) {
         if (!centres_out[v]) continue;
         const SlicView &s = b.v[v];

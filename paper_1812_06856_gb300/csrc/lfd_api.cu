@@ -1787,7 +1787,7 @@ lfd_status lfd_slic(lfd_ctx *ctx, int32_t n, const void *const *views, const int
     auto view_bytes = [&](int v, size_t &o_c, size_t &sz_c) {
         o_c = align_up(16 * cell_stride(v) * grid_w[v] * grid_h[v], 256);
         sz_c = align_up(20 * (size_t)grid_w[v] * grid_h[v], 256);
-        return o_c + 2 * sz_c + align_up(cell_stride(v) * grid_w[v] * grid_h[v], 256);
+        return o_c + 2 * sz_c + align_up(432 * (size_t)grid_w[v] * grid_h[v], 256);
     };
     for (int v = 0; v < n; v++) {
         if (width[v] < 1 || height[v] < 1 || width[v] > LFD_MAX_DIM || height[v] > LFD_MAX_DIM || grid_w[v] < 1 ||
@@ -1826,7 +1826,7 @@ lfd_status lfd_slic(lfd_ctx *ctx, int32_t n, const void *const *views, const int
             sv.lab = (float4 *)base;
             sv.centres = (float *)(base + o_c);
             sv.centres2 = (float *)(base + o_c + sz_c);
-            sv.code = (unsigned char *)(base + o_c + 2 * sz_c);
+            sv.sums = (long long *)(base + o_c + 2 * sz_c);
             sv.labels = labels_out[v];
             base += bytes;
             const double step = std::sqrt((double)sv.W * sv.H / ((double)sv.GW * sv.GH));

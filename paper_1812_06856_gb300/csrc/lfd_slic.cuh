@@ -9,11 +9,11 @@ namespace lfd {
 // one view of a SLIC segmentation
 struct SlicView {
     int W, H, GW, GH, fmt;
-    int stride;                      // entries of `lab` and `code` per cell (the largest cell, rounded up to 4)
+    int stride;                      // entries of `lab` per cell (the largest cell, rounded up to 4)
     long long pitch;                 // bytes per image row
     const void *img;
     float4 *lab;                     // [GW*GH][stride] CIELAB and position of a cell's pixels (scratch)
-    unsigned char *code;             // [GW*GH][stride] the pixels' picks among the 3x3 cells (scratch)
+    long long *sums;                 // [GW*GH][9][6] sums of a cell's pixels per centre of its 3x3 cells (scratch)
     int *labels;                     // [W*H] output
     float *centres, *centres2;       // [GW*GH][5] {L, a, b, x, y} (scratch, ping-pong)
 };
