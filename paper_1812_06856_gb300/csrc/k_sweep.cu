@@ -362,8 +362,8 @@ __device__ __forceinline__ void sweep_sp(const Workspace &w, const Consts &c, in
 // wavefronts, six of which a sample's 24-byte record needs.  Four warps share
 // a superpixel because one warp each (29 KB of shared memory per four) left
 // the gathers 28 KB of L1: 49.5 and 17.7 ms.  12 CTAs per SM at 40 registers:
-// 25.9 / 13.5 ms, 10 at 48: 26.3 / 13.6, 8 at 64: 26.2 / 13.8.  BS_LANES 24,
-// 48, 96: within 2 %.
+// 25.9 / 13.5 ms, 10 at 48: 26.3 / 13.6, 8 at 64: 26.2 / 13.8; two warps per
+// CTA: 44.2 / 21.6, eight: 27.7 / 13.7.  BS_LANES 24, 48, 96: within 2 %.
 constexpr int BS_LABELS = SWEEP_BOUNDED_LABELS;
 constexpr int BS_LANES = 48;        // labels left at which the lanes turn to pixels
 constexpr int BS_BATCH = 8;         // labels per round of that
