@@ -575,9 +575,15 @@ __device__ __forceinline__ uint2 views_inside(const SpShared &sh, const HypF &h,
 // stall it (4 x 640x480, 12-pixel perturbed superpixels: 2.9 ms of propagation
 // with a body per slot count, 1.5 rolled).  Superpixels of 225 to 256 pixels,
 // the 16 x 16 cells of regular grids, keep an unrolled body of their own (16 x
-// 1080p: 62.8 ms rolled, 55.2 unrolled).  Bound now by the gathers' latency
+// 1080p: 62.8 ms rolled, 55.2 unrolled), and superpixels of at most 128 pixels
+// have one without a loop, all of their gathers in flight together (one
+// iteration, 960x640, pitch 9, 4 views: 933 us rolled, 823; a batch of cold
+// light fields 41.0 -> 38.2 ms; the third body costs 1 % where the unrolled one
+// runs: 16 x 1080p 83.6 -> 84.7 ms a frame).  It is asked for first: the other
+// order gave 906 us, 39.5 and 84.3 ms.  Bound now by the gathers' latency
 // (issue 65 % of the cycles, long scoreboard the largest stall).
 constexpr int INSIDE_SLOTS = 4;   // slots per iteration of the rolled body
+constexpr int SHALLOW_SLOTS = 4;  // superpixels up to here have a body without a loop
 constexpr int UNROLLED_SLOTS = 8;
 
 // SL: 0 the rolled body, else an unrolled one for superpixels of SL slots
@@ -632,7 +638,10 @@ __device__ __forceinline__ ViewTerms view_term_inside(const Workspace &w, const 
         tail(act0, tx.x, ty.x, Nw.x, gp.x, val.x);
         tail(act1, tx.y, ty.y, Nw.y, gp.y, val.y);
     };
-    if constexpr (SL > 0) {
+    if constexpr (SL == SHALLOW_SLOTS) {                      // one to four slots: no loop
+        pair(0, lane < count, lane + 32 < count);
+        if (count > 64) pair(2, lane + 64 < count, lane + 96 < count);
+    } else if constexpr (SL > 0) {
 #pragma unroll
         for (int j = 0; j < SL; j += 2)
             pair(j, j + 1 < SL || lane + 32 * j < count, j + 1 < SL && (j + 2 < SL || lane + 32 * (j + 1) < count));
@@ -716,8 +725,9 @@ __device__ __noinline__ float2 eval_candidate(const Workspace &w, int src, float
     for (int k = 0; k < nnb; k++) {
         ViewTerms t = {0.f, 0.f, 0.f, 0u, 0u, 0u};            // no pixel in view: no terms
         if ((where.x >> (4 * k)) & 1u)
-            t = slots == UNROLLED_SLOTS ? view_term_inside<DOMAIN, AFF, UNROLLED_SLOTS>(w, sh, h, k, lane, count)
-                                        : view_term_inside<DOMAIN, AFF, 0>(w, sh, h, k, lane, count);
+            t = slots <= SHALLOW_SLOTS   ? view_term_inside<DOMAIN, AFF, SHALLOW_SLOTS>(w, sh, h, k, lane, count)
+                : slots == UNROLLED_SLOTS ? view_term_inside<DOMAIN, AFF, UNROLLED_SLOTS>(w, sh, h, k, lane, count)
+                                          : view_term_inside<DOMAIN, AFF, 0>(w, sh, h, k, lane, count);
         else if (!((where.y >> (4 * k)) & 1u)) t = view_term<DOMAIN, AFF>(w, sh, h, k, lane, slots, false);
         ec += t.Vi + t.Oi;
         if (cand_bound(sh, ec, (float)(nnb - 1 - k), h.es) < Ebest) return make_float2(-1.f, (float)(k + 1));
