@@ -36,6 +36,7 @@
 // are evaluated in FP32, which keeps the sub-pixel position exact to ~1e-6 px
 // and makes the nearest-pixel choice match an FP64 evaluation except within
 // that distance of a rounding boundary.
+#include "lfd_bounds.cuh"
 #include "lfd_sample.cuh"
 
 namespace lfd {
@@ -520,18 +521,14 @@ __device__ __forceinline__ ViewTerms view_term(const Workspace &w, const SpShare
 // Neighbour views in which every pixel of the superpixel lands inside the
 // image, in front of both cameras, under hypothesis h (x: bit 4 k for view k),
 // or outside it (y).  Lane 4 k + c tests corner c of the offsets' box in view
-// k; inverse depth and homogeneous coordinate are affine in the offset, and a
-// homography takes a box in front of the camera into the hull of its corners,
-// so the corners decide for all pixels.  Margins: 0.1 px of the half pixel to
-// the window edge (a position's rounding is below 0.01 px up to 32767 px),
-// 1e-5 of the summed magnitudes for the sign of the inverse depth, a factor 4
-// for the range of the homogeneous coordinate.
+// k (corner_sides); inverse depth and homogeneous coordinate are affine in the
+// offset, so the corners decide for all pixels.  1e-5 of the summed magnitudes
+// covers the sign of the inverse depth.
 template <bool AFF>
 __device__ __forceinline__ uint2 views_inside(const SpShared &sh, const HypF &h, int nnb, float xy, int lane)
 {
     const int k = lane >> 2;
-    bool in = false, front = false;
-    float x = 0.f, y = 0.f, xe = 0.f, ye = 0.f;
+    CornerSides c = {false, false, false, false, false};
     if (k < nnb) {
         const SpView &sv = sh.view[k];
         const float du = (lane & 1) ? sh.bx1 : sh.bx0, dv = (lane & 2) ? sh.by1 : sh.by0;
@@ -541,15 +538,9 @@ __device__ __forceinline__ uint2 views_inside(const SpShared &sh, const HypF &h,
                               fmaf(fmaf(sv.Dx, h.g1, sv.Pp01), dv, fmaf(sv.Dx, h.dgr, sv.Ex)));
         const float ey = fmaf(fmaf(sv.Dy, h.g0, sv.Pp10), du,
                               fmaf(fmaf(sv.Dy, h.g1, sv.Pp11), dv, fmaf(sv.Dy, h.dgr, sv.Ey)));
-        const float r = rcp_approx(Nw);
-        x = (float)(sv.xa_m + 0x4B400000) + ex * r;
-        y = (float)(sv.ya_m + 0x4B400000) + ey * r;
-        xe = (float)sv.Wi - 0.5f;
-        ye = (float)sv.Hi - 0.5f;
+        c = corner_sides(ex, ey, rcp_approx(Nw), Nw, hw, sv.xa_m + 0x4B400000, sv.ya_m + 0x4B400000, sv.Wi, sv.Hi);
         const float a = h.g0 * du, b = h.g1 * dv, gp = a + b + h.gr;
-        front = hw > 0.f && Nw > 0.25f * hw && Nw < 4.f * hw;
-        in = front && xy == 1.f && gp > 1e-5f * (fabsf(a) + fabsf(b) + fabsf(h.gr)) && x >= -0.4f && x <= xe - 0.1f &&
-             y >= -0.4f && y <= ye - 0.1f;
+        c.in = c.in && xy == 1.f && gp > 1e-5f * (fabsf(a) + fabsf(b) + fabsf(h.gr));
     }
     auto all4 = [](bool p) {
         unsigned m = __ballot_sync(0xffffffffu, p);
@@ -557,9 +548,8 @@ __device__ __forceinline__ uint2 views_inside(const SpShared &sh, const HypF &h,
         return m & (m >> 1);
     };
     uint2 m;
-    m.x = all4(in);
-    m.y = all4(front && x < -0.6f) | all4(front && x > xe + 0.1f) | all4(front && y < -0.6f) |
-          all4(front && y > ye + 0.1f);
+    m.x = all4(c.in);
+    m.y = all4(c.x0) | all4(c.x1) | all4(c.y0) | all4(c.y1);
     return m;
 }
 

@@ -1,0 +1,127 @@
+"""The samples taken without a window test stay inside the view: random
+hypotheses that land on the image border, far outside the anchor of the
+current plane and near the neighbour's principal plane, through the corner
+test that admits them (csrc/lfd_bounds.cuh, compiled for the host)."""
+import ctypes
+import os
+import subprocess
+
+import pytest
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+CSRC = os.path.join(ROOT, "paper_1812_06856_gb300", "csrc")
+
+SOURCE = r"""
+#include <cmath>
+#include <cstdint>
+#include <random>
+#include "lfd_bounds.cuh"
+using namespace lfd;
+
+// a rotation of the neighbour by angle a about y and b about x
+static void pair(double f, int W, int H, double a, double b, const double t[3], double P[9], double q[3])
+{
+    const double R[9] = {cos(a), 0, sin(a), sin(a) * sin(b), cos(b), -cos(a) * sin(b), -sin(a) * cos(b), sin(b), cos(a) * cos(b)};
+    const double K[9] = {f, 0, (W - 1) / 2.0, 0, f, (H - 1) / 2.0, 0, 0, 1};
+    const double Ki[9] = {1 / f, 0, -K[2] / f, 0, 1 / f, -K[5] / f, 0, 0, 1};
+    double KR[9];
+    for (int i = 0; i < 3; i++)
+        for (int j = 0; j < 3; j++) {
+            KR[3 * i + j] = 0;
+            for (int k = 0; k < 3; k++) KR[3 * i + j] += K[3 * i + k] * R[3 * k + j];
+        }
+    for (int i = 0; i < 3; i++) {
+        q[i] = 0;
+        for (int k = 0; k < 3; k++) q[i] += K[3 * i + k] * t[k];
+        for (int j = 0; j < 3; j++) {
+            P[3 * i + j] = 0;
+            for (int k = 0; k < 3; k++) P[3 * i + j] += KR[3 * i + k] * Ki[3 * k + j];
+        }
+    }
+}
+
+static float as_float(uint32_t u) { float f; __builtin_memcpy(&f, &u, 4); return f; }
+static uint32_t as_bits(float f) { uint32_t u; __builtin_memcpy(&u, &f, 4); return u; }
+// 1 / x within one unit of the last place, as the device's estimate
+static float rcp(float x, int ulp) { return as_float(as_bits(1.0f / x) + ulp); }
+
+// out: boxes admitted as inside, as outside, and those of each with a pixel that is not
+extern "C" void refine_boxes(uint64_t seed, long trials, long out[4])
+{
+    std::mt19937_64 g(seed);
+    auto U = [&](double lo, double hi) { return lo + (hi - lo) * (g() >> 11) * 0x1p-53; };
+    for (int k = 0; k < 4; k++) out[k] = 0;
+    const int sizes[4][2] = {{640, 480}, {1920, 1080}, {3840, 2160}, {32767, 400}};
+    for (long it = 0; it < trials; it++) {
+        const int *sz = sizes[g() & 3], W = sz[0], H = sz[1], side = 1 + (int)(g() % 24);
+        const double f = W * U(0.5, 1.2), rs = U(0.01, 10.0);
+        const double t[3] = {U(-2, 2), U(-0.2, 0.2), U(-2, 2)};
+        double P[9], q[3];
+        pair(f, W, H, U(-1.5, 1.5), U(-0.1, 0.1), t, P, q);
+        const int rx = (int)U(0, W), ry = (int)U(0, H);
+        double pr[3];
+        for (int k = 0; k < 3; k++) pr[k] = P[3 * k] * rx + P[3 * k + 1] * ry + P[3 * k + 2];
+        // anchor of the current plane: homogeneous coordinate from 1e-5 to 1; candidate: its own
+        // position on the left or right border
+        const double hwa = exp(U(-11.5, 0)), za = (hwa - pr[2]) / q[2];
+        const double edge = (g() & 1 ? W - 0.5 : -0.5) + U(-1.2, 1.2);
+        const double z1 = (edge * pr[2] - pr[0]) / (q[0] - edge * q[2]);
+        if (!(z1 > 0) || !(za > 0) || z1 > 100 || za > 100) continue;
+        const double g0 = U(-1, 1) * z1 / W, g1 = U(-1, 1) * z1 / W;
+        const double hx = q[0] * za + pr[0], hy = q[1] * za + pr[1], hw = q[2] * za + pr[2];
+        const double xa = fmin(fmax(floor(hx / hw), -1048576.0), 1048576.0), ya = fmin(fmax(floor(hy / hw), -1048576.0), 1048576.0);
+        const float dgr = (float)(z1 - za), g0f = (float)g0, g1f = (float)g1;
+        const float hwc = fmaf((float)(q[2] * rs), dgr, (float)(hw * rs));
+        const float cx = fmaf((float)((q[0] - xa * q[2]) * rs), dgr, (float)((hx - xa * hw) * rs));
+        const float cy = fmaf((float)((q[1] - ya * q[2]) * rs), dgr, (float)((hy - ya * hw) * rs));
+        const float dx = (float)((q[0] - xa * q[2]) * rs), dy = (float)((q[1] - ya * q[2]) * rs), qw = (float)(q[2] * rs);
+        const float b0 = fmaf(dx, g0f, (float)((P[0] - xa * P[6]) * rs)), b1 = fmaf(dx, g1f, (float)((P[1] - xa * P[7]) * rs));
+        const float c0 = fmaf(dy, g0f, (float)((P[3] - ya * P[6]) * rs)), c1 = fmaf(dy, g1f, (float)((P[4] - ya * P[7]) * rs));
+        const float a20 = fmaf(qw, g0f, (float)(P[6] * rs)), a21 = fmaf(qw, g1f, (float)(P[7] * rs));
+        const int lo = -(int)(g() % (side + 1)), hi = lo + side;
+        bool in = true, x0 = true, x1 = true, y0 = true, y1 = true;
+        for (int c = 0; c < 4; c++) {
+            const float du = (float)(c & 1 ? hi : lo), dv = (float)(c & 2 ? hi : lo);
+            const float Nw = fmaf(a20, du, fmaf(a21, dv, hwc));
+            const float ex = fmaf(b0, du, fmaf(b1, dv, cx)), ey = fmaf(c0, du, fmaf(c1, dv, cy));
+            const CornerSides s = corner_sides(ex, ey, rcp(Nw, (int)(g() % 3) - 1), Nw, hwc, (int)xa, (int)ya, W, H);
+            in = in && s.in;
+            x0 = x0 && s.x0; x1 = x1 && s.x1; y0 = y0 && s.y0; y1 = y1 && s.y1;
+        }
+        const bool off = x0 || x1 || y0 || y1;
+        if (!in && !off) continue;
+        out[in ? 0 : 1]++;
+        bool wrong = false;
+        for (int v = lo; v <= hi; v++)
+            for (int u = lo; u <= hi; u++) {
+                const float du = (float)u, dv = (float)v, Nw = fmaf(a20, du, fmaf(a21, dv, hwc));
+                const float ex = fmaf(b0, du, fmaf(b1, dv, cx)), ey = fmaf(c0, du, fmaf(c1, dv, cy));
+                const float r = rcp(Nw, (int)(g() % 3) - 1);
+                const float tx = fmaf(ex, r, 12582912.f), ty = fmaf(ey, r, 12582912.f);      // 1.5 * 2^23: nearest integer
+                const uint32_t ix = as_bits(tx) - 0x4B400000u + (uint32_t)(int)xa, iy = as_bits(ty) - 0x4B400000u + (uint32_t)(int)ya;
+                const bool pixel = Nw > 0.f && ix < (uint32_t)W && iy < (uint32_t)H;
+                wrong = wrong || pixel != in;
+            }
+        if (wrong) out[in ? 2 : 3]++;
+    }
+}
+"""
+
+
+@pytest.fixture(scope="module")
+def probe(tmp_path_factory):
+    d = tmp_path_factory.mktemp("inside")
+    src, lib = d / "probe.cpp", d / "probe.so"
+    src.write_text(SOURCE)
+    subprocess.check_call(["g++", "-O2", "-std=c++17", "-ffp-contract=off", "-fPIC", "-shared", "-I", CSRC, "-o", str(lib),
+                           str(src)])
+    return ctypes.CDLL(str(lib))
+
+
+@pytest.mark.parametrize("seed", [1, 2, 3])
+def test_boxes_of_the_refinement_are_on_the_side_they_are_taken_for(probe, seed):
+    out = (ctypes.c_long * 4)()
+    probe.refine_boxes(ctypes.c_uint64(seed), ctypes.c_long(4_000_000), out)
+    inside, outside, wrong_in, wrong_out = out
+    assert inside > 1000 and outside > 1000
+    assert (wrong_in, wrong_out) == (0, 0)
