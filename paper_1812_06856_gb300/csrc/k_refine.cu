@@ -386,11 +386,9 @@ __device__ __forceinline__ void sample_tail(const ViewK &K, bool act, float Nw, 
     // an exact .5 as a rounding boundary where either pixel is admissible).
     // The point lies in view i iff that pixel does (-1/2 <= x < W - 1/2);
     // out-of-range or non-finite offsets give out-of-range integers.
-    const int ix = __float_as_int(tx) + K.xa_m;
-    const int iy = __float_as_int(ty) + K.ya_m;
-    const bool ok = act && (gp > 0.f) && (!CHECKW || Nw > 0.f) && ((unsigned)ix < (unsigned)K.Wi) &&
-                    ((unsigned)iy < (unsigned)K.Hi);
-    const int idx = ok ? iy * K.Wi + ix : 0;                     // in-bounds address either way
+    const unsigned ix = pixel_coord(tx, K.xa_m), iy = pixel_coord(ty, K.ya_m);
+    const bool ok = act && (gp > 0.f) && (!CHECKW || Nw > 0.f) && ix < (unsigned)K.Wi && iy < (unsigned)K.Hi;
+    const unsigned idx = ok ? iy * (unsigned)K.Wi + ix : 0u;     // in-bounds address either way
     const float4 c = __ldg(K.map + idx);                         // {colour of the superpixel hit, depth value}
     const float tw = c.w;
     const float2 drg = fsub2(make_float2(c.x, c.y), make_float2(cr, cg));   // red, green as a packed pair
@@ -589,15 +587,15 @@ __device__ __forceinline__ ViewTerms view_term_inside(const Workspace &w, const 
     const float2 G0 = dup2(h.g0), G1 = dup2(h.g1), GR = dup2(h.gr), M = dup2(ROUND_MAGIC);
     const float2 A20 = dup2(fmaf(sv.qw, h.g0, sv.P20)), A21 = dup2(fmaf(sv.qw, h.g1, sv.P21)), HW = dup2(hw);
     const float cr = sh.S.cr, cg = sh.S.cg, cb = sh.S.cb;
-    const int Wi = sv.Wi, base = sv.ya_m * Wi + sv.xa_m;      // modulo 2^32
+    const int Wi = sv.Wi;
+    const unsigned base = pixel_base(sv.xa_m, sv.ya_m, Wi);
     const float4 *map = sv.map;
     const float2 Raff = dup2(AFF ? rcp_approx(hw) : 0.f);
     float sw = 0.f, sg = 0.f;
     unsigned nx = 0;
     bool anyY = false;
     auto tail = [&](bool act, float tx, float ty, float Nw, float gp, float val0) {
-        const int idx = __float_as_int(ty) * Wi + (__float_as_int(tx) + base);
-        const float4 c = __ldg(map + idx);
+        const float4 c = __ldg(map + pixel_index(tx, ty, Wi, base));
         const float2 drg = fsub2(make_float2(c.x, c.y), make_float2(cr, cg));
         const float2 d2 = fmul2(drg, drg);
         const float db = c.z - cb;

@@ -3,6 +3,7 @@
 // operation).
 #pragma once
 #include <math.h>
+#include <string.h>
 #ifdef __CUDACC__
 #define LFD_HD __host__ __device__ __forceinline__
 #else
@@ -50,6 +51,31 @@ LFD_HD CornerSides corner_sides(float ex, float ey, float r, float Nw, float hw,
     c.y0 = fit && y < lo;
     c.y1 = fit && y > ye;
     return c;
+}
+
+// Nearest pixels by adding 1.5 * 2^23: t carries the offset from the anchor
+// pixel in its low bits, a_m is the anchor pixel minus the bits of 1.5 * 2^23.
+// Modulo 2^32: an offset out of range (|f| >= 2^22, infinite, NaN) gives a
+// coordinate that no view has.
+LFD_HD unsigned float_bits(float t)
+{
+#ifdef __CUDA_ARCH__
+    return __float_as_uint(t);
+#else
+    unsigned u;
+    memcpy(&u, &t, 4);
+    return u;
+#endif
+}
+
+LFD_HD unsigned pixel_coord(float t, int a_m) { return float_bits(t) + (unsigned)a_m; }
+
+// index of an inside pixel in a view of width Wi, base = pixel_base(xa_m, ya_m, Wi)
+LFD_HD unsigned pixel_base(int xa_m, int ya_m, int Wi) { return (unsigned)ya_m * (unsigned)Wi + (unsigned)xa_m; }
+
+LFD_HD unsigned pixel_index(float tx, float ty, int Wi, unsigned base)
+{
+    return float_bits(ty) * (unsigned)Wi + (float_bits(tx) + base);
 }
 
 }  // namespace lfd

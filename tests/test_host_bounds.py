@@ -125,3 +125,40 @@ def test_boxes_of_the_refinement_are_on_the_side_they_are_taken_for(probe, seed)
     inside, outside, wrong_in, wrong_out = out
     assert inside > 1000 and outside > 1000
     assert (wrong_in, wrong_out) == (0, 0)
+
+
+INDEX = r"""
+#include <cstdio>
+#include <random>
+#include "lfd_bounds.cuh"
+using namespace lfd;
+
+int main()
+{
+    std::mt19937_64 g(1);
+    for (int it = 0; it < 2000000; it++) {
+        const int W = 1 + (int)(g() % 32767), H = 1 + (int)(g() % 32767), x = (int)(g() % W), y = (int)(g() % H);
+        const int xa = (int)(g() % 2097153) - 1048576, ya = (int)(g() % 2097153) - 1048576;
+        const float tx = (float)(x - xa) + 12582912.f, ty = (float)(y - ya) + 12582912.f;
+        const int xm = xa - 0x4B400000, ym = ya - 0x4B400000;
+        if (pixel_coord(tx, xm) != (unsigned)x || pixel_coord(ty, ym) != (unsigned)y) return 1;
+        if (pixel_index(tx, ty, W, pixel_base(xm, ym, W)) != (unsigned)(y * W + x)) return 2;
+        // an offset out of range is no pixel of any view
+        unsigned bits = (unsigned)g();
+        float f;
+        memcpy(&f, &bits, 4);
+        if (!(fabsf(f) < 4194304.f) && pixel_coord(f + 12582912.f, xm) < 32767u) return 3;
+    }
+    printf("ok");
+    return 0;
+}
+"""
+
+
+def test_pixel_indices_are_taken_modulo_two_to_the_32(tmp_path):
+    (tmp_path / "index.cpp").write_text(INDEX)
+    exe = tmp_path / "index"
+    subprocess.check_call(["g++", "-O1", "-std=c++17", "-ffp-contract=off", "-fsanitize=signed-integer-overflow",
+                           "-fsanitize-undefined-trap-on-error", "-I", CSRC, "-o", str(exe), str(tmp_path / "index.cpp")])
+    r = subprocess.run([str(exe)], capture_output=True, text=True)
+    assert (r.returncode, r.stdout) == (0, "ok")
