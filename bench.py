@@ -65,7 +65,7 @@ FP32_LANES_PER_SM = 128
 
 KERNEL_SOURCES = {
     "k_propagate": ["k_refine.cu", "lfd_bounds.cuh", "lfd_sample.cuh", "lfd_internal.cuh"],
-    "k_sweep": ["k_sweep.cu", "lfd_sample.cuh", "lfd_internal.cuh"],
+    "k_sweep": ["k_sweep.cu", "lfd_bounds.cuh", "lfd_sample.cuh", "lfd_internal.cuh"],
 }
 
 

@@ -25,6 +25,7 @@
 // world frame the label also scales the pixel terms: 6 FP32 FMAs per sample.
 #include <type_traits>
 
+#include "lfd_bounds.cuh"
 #include "lfd_sample.cuh"
 
 namespace lfd {
@@ -465,25 +466,8 @@ struct LabelView {
         if (!ok) return false;
         if (PF == PF_SHIFT)
             return ox + x0 >= 0 && ox + x1 <= sp.Wi - 1 && oy + y0 >= 0 && oy + y1 <= sp.Hi - 1;
-        // corners of the box, with a margin for the rounding of a sample's
-        // position (below 0.01 px up to 32767 px); the homography maps a box in
-        // front of the camera into the hull of its corners
-        bool in = true;
-        float wmin = INFINITY, wmax = -INFINITY;
-#pragma unroll
-        for (int c = 0; c < 4; c++) {
-            const float du = (float)((c & 1) ? x1 : x0), dv = (float)((c & 2) ? y1 : y0);
-            float r = cw;
-            if (PF == PF_GENERAL) {
-                const float W = fmaf(sp.a20, du, fmaf(sp.a21, dv, cw));
-                wmin = fminf(wmin, W);
-                wmax = fmaxf(wmax, W);
-                r = rcp_approx(W);
-            }
-            const float x = fmaf(sp.a00, du, fmaf(sp.a01, dv, cx)) * r, y = fmaf(sp.a10, du, fmaf(sp.a11, dv, cy)) * r;
-            in = in && x >= -0.45f && x <= (float)sp.Wi - 0.55f && y >= -0.45f && y <= (float)sp.Hi - 0.55f;
-        }
-        return in && (PF == PF_AFFINE || wmin > 1e-3f * wmax);
+        return box_inside(PF == PF_GENERAL, sp.a00, sp.a01, sp.a10, sp.a11, sp.a20, sp.a21, cx, cy, cw, sp.Wi, sp.Hi,
+                          x0, x1, y0, y1);
     }
 
     template <typename C>

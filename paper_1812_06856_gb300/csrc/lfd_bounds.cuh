@@ -12,6 +12,18 @@
 
 namespace lfd {
 
+// 1 / x to one unit of the last place (the device's estimate)
+LFD_HD float reciprocal(float x)
+{
+#ifdef __CUDA_ARCH__
+    float y;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+#else
+    return 1.0f / x;
+#endif
+}
+
 // ---------------------------------------------------------------------------
 // window tests of energy samples: nearest pixel, positions relative to an anchor
 // ---------------------------------------------------------------------------
@@ -76,6 +88,48 @@ LFD_HD unsigned pixel_base(int xa_m, int ya_m, int Wi) { return (unsigned)ya_m *
 LFD_HD unsigned pixel_index(float tx, float ty, int Wi, unsigned base)
 {
     return float_bits(ty) * (unsigned)Wi + (float_bits(tx) + base);
+}
+
+// ---------------------------------------------------------------------------
+// window tests of sweep samples: bilinear, positions in image coordinates
+// ---------------------------------------------------------------------------
+//
+// A sample's position is X / Z with X = c + (a0 du + a1 dv), Z likewise (or Z
+// constant): near the neighbour's principal plane, or far from the
+// superpixel's anchor, terms much larger than X cancel in it.  With MX and MZ
+// the largest sums of the terms' magnitudes over the box and Z >= zmin, one
+// evaluation errs by at most 3 u MX / zmin + |x| (3 u MZ / zmin + 3 u), two of
+// them by 12 u (MX + W MZ) / zmin, which is below BOX_MARGIN (0.215 px) where
+// MX + W MZ <= BOX_REACH zmin.  A sample that is admitted so reads the texture
+// from the entries -1 to W - 1 that the view has.
+constexpr float BOX_REACH = 3e5f, BOX_MARGIN = 0.25f;
+
+// the offsets [x0, x1] x [y0, y1] all sample inside a Wi x Hi view.  general:
+// cz is the anchor's homogeneous coordinate; else Z is constant, cz = 1 / Z
+LFD_HD bool box_inside(bool general, float a00, float a01, float a10, float a11, float a20, float a21, float cx,
+                       float cy, float cz, int Wi, int Hi, int x0, int x1, int y0, int y1)
+{
+    const float mu = fmaxf(fabsf((float)x0), fabsf((float)x1)), mv = fmaxf(fabsf((float)y0), fabsf((float)y1));
+    const float xe = (float)Wi - 0.5f - BOX_MARGIN, ye = (float)Hi - 0.5f - BOX_MARGIN;
+    float zmin = INFINITY;
+    bool in = true;
+    for (int c = 0; c < 4; c++) {
+        const float du = (float)((c & 1) ? x1 : x0), dv = (float)((c & 2) ? y1 : y0);
+        const float X = fmaf(a00, du, fmaf(a01, dv, cx)), Y = fmaf(a10, du, fmaf(a11, dv, cy));
+        float r = cz;
+        if (general) {
+            const float Z = fmaf(a20, du, fmaf(a21, dv, cz));
+            zmin = fminf(zmin, Z);
+            r = reciprocal(Z);
+        }
+        const float x = X * r, y = Y * r;
+        in = in && x >= BOX_MARGIN - 0.5f && x <= xe && y >= BOX_MARGIN - 0.5f && y <= ye;
+    }
+    const float MX = fmaf(fabsf(a00), mu, fmaf(fabsf(a01), mv, fabsf(cx)));
+    const float MY = fmaf(fabsf(a10), mu, fmaf(fabsf(a11), mv, fabsf(cy)));
+    if (!general) return in && MX * cz + (float)Wi <= BOX_REACH && MY * cz + (float)Hi <= BOX_REACH;
+    const float MZ = fmaf(fabsf(a20), mu, fmaf(fabsf(a21), mv, fabsf(cz)));
+    return in && zmin > 0.f && fmaf((float)Wi, MZ, MX) <= BOX_REACH * zmin && fmaf((float)Hi, MZ, MY) <= BOX_REACH * zmin;
 }
 
 }  // namespace lfd

@@ -1,7 +1,7 @@
 """The samples taken without a window test stay inside the view: random
 hypotheses that land on the image border, far outside the anchor of the
 current plane and near the neighbour's principal plane, through the corner
-test that admits them (csrc/lfd_bounds.cuh, compiled for the host)."""
+tests that admit them (csrc/lfd_bounds.cuh, compiled for the host)."""
 import ctypes
 import os
 import subprocess
@@ -105,6 +105,55 @@ extern "C" void refine_boxes(uint64_t seed, long trials, long out[4])
         if (wrong) out[in ? 2 : 3]++;
     }
 }
+
+// chunks of a superpixel in one neighbour view, near its border and its principal plane;
+// out: boxes admitted, and those with a sample outside the window
+extern "C" void sweep_boxes(uint64_t seed, long trials, long out[2])
+{
+    std::mt19937_64 g(seed);
+    auto U = [&](double lo, double hi) { return lo + (hi - lo) * (g() >> 11) * 0x1p-53; };
+    out[0] = out[1] = 0;
+    const int sizes[4][2] = {{640, 480}, {1920, 1080}, {3840, 2160}, {32767, 400}};
+    for (long it = 0; it < trials; it++) {
+        const int *sz = sizes[g() & 3], W = sz[0], H = sz[1];
+        const double f = W * U(0.5, 1.2), t[3] = {U(-2, 2), U(-0.2, 0.2), U(-2, 0)};
+        const bool general = g() & 3;
+        double P[9], q[3];
+        pair(f, W, H, general ? U(-1.5, 1.5) : 0.0, general ? U(-0.1, 0.1) : 0.0, t, P, q);
+        // the chunk's box, at any offset from the superpixel's anchor
+        const int far = 1 << (g() % 12), x0 = (int)U(-far, far), y0 = (int)U(-far, far), w = (int)(g() % 12), h = (int)(g() % 12);
+        const double px = U(0, W), py = U(0, H);
+        const int rx = (int)px - x0, ry = (int)py - y0;
+        double pr[3], pp[3];
+        for (int k = 0; k < 3; k++) {
+            pr[k] = P[3 * k] * rx + P[3 * k + 1] * ry + P[3 * k + 2];
+            pp[k] = P[3 * k] * (rx + x0) + P[3 * k + 1] * (ry + y0) + P[3 * k + 2];
+        }
+        // a camera that has the box's first pixel on the window's edge, at 1e-4 to 1 of its depth
+        const double edge = (g() & 1 ? W - 0.5 : -0.5) + U(-0.6, 0.6), z = U(0.1, 2), near = exp(U(-9, 0)), at = U(0, H);
+        if (general) {
+            q[0] = (edge * near - pp[0]) / z;
+            q[1] = (at * near - pp[1]) / z;
+            q[2] = (near - pp[2]) / z;
+        }
+        const float a00 = (float)P[0], a01 = (float)P[1], a10 = (float)P[3], a11 = (float)P[4], a20 = (float)P[6], a21 = (float)P[7];
+        const float cx = (float)(z * q[0] + pr[0]), cy = (float)(z * q[1] + pr[1]), cw = (float)(z * q[2] + pr[2]);
+        if (!general && !(cw > 0.f)) continue;
+        const float rc = general ? cw : rcp(cw, (int)(g() % 3) - 1);
+        if (!box_inside(general, a00, a01, a10, a11, a20, a21, cx, cy, rc, W, H, x0, x0 + w, y0, y0 + h)) continue;
+        out[0]++;
+        bool wrong = false;
+        for (int v = y0; v <= y0 + h; v++)
+            for (int u = x0; u <= x0 + w; u++) {
+                const float fu = (float)u, fv = (float)v;
+                const float A = fmaf(a00, fu, a01 * fv), B = fmaf(a10, fu, a11 * fv), wz = fmaf(a20, fu, a21 * fv) + cw;
+                const float r = general ? rcp(wz, (int)(g() % 3) - 1) : rc, x = (A + cx) * r, y = (B + cy) * r;
+                wrong = wrong || (general && !(wz > 0.f)) ||
+                        !(x >= -0.5f && x < (float)W - 0.5f && y >= -0.5f && y < (float)H - 0.5f);
+            }
+        out[1] += wrong;
+    }
+}
 """
 
 
@@ -162,3 +211,10 @@ def test_pixel_indices_are_taken_modulo_two_to_the_32(tmp_path):
                            "-fsanitize-undefined-trap-on-error", "-I", CSRC, "-o", str(exe), str(tmp_path / "index.cpp")])
     r = subprocess.run([str(exe)], capture_output=True, text=True)
     assert (r.returncode, r.stdout) == (0, "ok")
+
+
+@pytest.mark.parametrize("seed", [1, 2, 3])
+def test_boxes_of_the_sweep_are_inside(probe, seed):
+    out = (ctypes.c_long * 2)()
+    probe.sweep_boxes(ctypes.c_uint64(seed), ctypes.c_long(4_000_000), out)
+    assert out[0] > 1000 and out[1] == 0
