@@ -403,15 +403,6 @@ struct BoundedShared {
     SweepPair pair[LFD_MAXN];
 };
 
-// relative bound of the difference between an FP32 sum of the n * nnb
-// non-negative samples in k_sweep's order (chunks of up to 128 * nnb samples
-// one after another, then the chunk sums) or the order of the lane sums here,
-// and the exact sum: one rounding of 2^-24 per addition, doubled
-__device__ __forceinline__ float sweep_eps(int n, int nnb)
-{
-    return (float)(SWEEP_CHUNK * nnb + n / SWEEP_CHUNK + 96) * 1.2e-7f;
-}
-
 // a label's projection into one neighbour view, and its samples there
 template <int FMT, int PF>
 struct LabelView {
@@ -619,7 +610,7 @@ __device__ __forceinline__ void bounded_sweep_sp(const Workspace &w, int gs, Bou
         sh.taken = 0;
     }
 
-    const float eps = sweep_eps(n, nnb);
+    const float eps = sweep_eps(n, nnb, SWEEP_CHUNK);
     int K = L, best_k = -1;
     unsigned long long taken = 0;            // per warp (lane 0's count is added up)
     bool bounded = false;                    // B is known

@@ -132,4 +132,20 @@ LFD_HD bool box_inside(bool general, float a00, float a01, float a10, float a11,
     return in && zmin > 0.f && fmaf((float)Wi, MZ, MX) <= BOX_REACH * zmin && fmaf((float)Hi, MZ, MY) <= BOX_REACH * zmin;
 }
 
+// ---------------------------------------------------------------------------
+// sums of a label's costs in two orders
+// ---------------------------------------------------------------------------
+//
+// Relative bound of the difference between two FP32 sums of the n * nnb
+// non-negative samples of a label.  In the full sweep's order a sample goes
+// through up to chunk * nnb additions of its chunk and one per chunk; in the
+// order of the lanes (incumbent and last labels) through n / chunk * nnb of
+// its lane, and fewer than 16 of the lanes and warps.  One rounding of u per
+// addition in either order, doubled.
+LFD_HD float sweep_eps(int n, int nnb, int chunk)
+{
+    const float chunks = (float)(n / chunk + 1);
+    return ((float)(chunk * nnb) + chunks * (float)(nnb + 1) + 96.f) * 1.2e-7f;
+}
+
 }  // namespace lfd

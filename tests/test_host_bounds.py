@@ -154,6 +154,8 @@ extern "C" void sweep_boxes(uint64_t seed, long trials, long out[2])
         out[1] += wrong;
     }
 }
+
+extern "C" float bound_of_sums(int n, int nnb) { return sweep_eps(n, nnb, 128); }
 """
 
 
@@ -218,3 +220,15 @@ def test_boxes_of_the_sweep_are_inside(probe, seed):
     out = (ctypes.c_long * 2)()
     probe.sweep_boxes(ctypes.c_uint64(seed), ctypes.c_long(4_000_000), out)
     assert out[0] > 1000 and out[1] == 0
+
+
+@pytest.mark.parametrize("nnb", [1, 2, 4, 8])
+@pytest.mark.parametrize("n", [1, 127, 128, 256, 4096, 22_000, 65_536, 1 << 20, 1 << 24, (1 << 30) - 1])
+def test_bound_of_sums_covers_every_addition(probe, n, nnb):
+    """One rounding of 2^-24 for each addition a sample goes through: up to 128 nnb of its chunk and one per chunk in
+    the full sweep's order; nnb per chunk of 128 pixels in a lane, 4 slots, 5 steps of a butterfly and 4 warps in the
+    other."""
+    probe.bound_of_sums.restype = ctypes.c_float
+    chunks = -(-n // 128)
+    additions = (128 * nnb + chunks) + (chunks * nnb + 4 + 5 + 4)
+    assert probe.bound_of_sums(n, nnb) >= additions * 2.0 ** -24
