@@ -308,7 +308,9 @@ typedef struct {
                                   Needs a non-default stream. */
     int32_t sweep_threads;     /* 128 or 256 (0 = 256): labels scored in parallel per superpixel by a full
                                   sweep; persistent sweeps of up to 256 labels drop labels that can no
-                                  longer win and use CTAs of 128 threads */
+                                  longer win and use CTAs of 128 threads, unless the light fields'
+                                  superpixels are so small, or so few and large, that a full sweep
+                                  is the faster one */
     int32_t sweep_persistent;  /* 1: persistent sweep CTAs take superpixels from a queue ordered
                                   by size (pixel-slot class ceil(n/32)), largest first */
     int32_t prop_blocks;       /* 7 or 8 (0 = 8); both run 7 resident propagation CTAs per SM, the

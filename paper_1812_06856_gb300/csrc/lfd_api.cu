@@ -248,6 +248,7 @@ struct lfd_ctx {
     uint64_t tuned_sig = 0;
     // sweep launches: superpixels of label-count class c at order_sweep[cls_base[c] ..+ cls_count[c])
     int cls_base[NSCLASS] = {}, cls_count[NSCLASS] = {};
+    bool cls_bounded[NSCLASS] = {};  // the class takes the bounded sweep (bounded_pays)
 };
 
 namespace {
@@ -566,6 +567,33 @@ lfd_status plan_workspace(lfd_ctx *ctx, int n, const lfd_lightfield *lfs)
     return LFD_OK;
 }
 
+// Whether a sweep class (superpixels S of px pixels in all, up to L labels and
+// nnb neighbour views, pair form pf) is swept with bounds: it costs a
+// superpixel a CTA of 128 threads, a barrier per chunk and view, and a last
+// stage with 32 lanes on the pixels.  The full sweep, a thread per label, is
+// the faster one (us, bounded against full; 640x480, 3 neighbour views, grid
+// or arc of cameras, RGBA8, unless another size is named)
+// - for superpixels of a few pixels and views: of 16 pixels with 64 labels 1076
+//   and 971 (grid), 1561 and 1330 (arc); of 25 793 and 824, 1176 and 1291;
+// - without a common shift (general pairs) also below 128 pixels and views
+//   together where the label count leaves passes or the last stage uneven: of
+//   25 pixels with 33 labels 1770 and 1097, 160 labels 2228 and 1391; of 64
+//   pixels 988 and 1039, 1414 and 1264;
+// - above 128 labels where large superpixels are too few to fill a wave: on the
+//   grid 320 of 4096 pixels, 256 labels, 4680 and 3526, 48 of 25600 34159 and
+//   20314; 1280x720, 8 neighbour views, 936 of 9216 47498 and 41527, 1980 of
+//   4096 24417 and 28888; on the arc 768 of 1600 3568 and 3158, 1200 of 1024
+//   with 160 labels 2506 and 1933.
+bool bounded_pays(int pf, int L, int nnb, long long px, int S, int sms)
+{
+    if (L > SWEEP_BOUNDED_LABELS) return false;
+    const long long mean = px / std::max(S, 1);
+    if (mean * nnb < 64) return false;
+    if (pf == 0 && (L <= 48 || L > 128) && mean * nnb < 128) return false;
+    if (L > 128 && mean >= (pf == 0 ? 1000 : 2000) && S <= sms * (pf == 0 ? 13 : 7)) return false;
+    return true;
+}
+
 // Host half of binding n light fields: validation, workspace, records staged in
 // pinned memory.  Nothing is enqueued.
 lfd_status plan_input(lfd_ctx *ctx, int n, const lfd_lightfield *lfs, const lfd_params *ps, bool host_mem)
@@ -722,6 +750,15 @@ lfd_status plan_input(lfd_ctx *ctx, int n, const lfd_lightfield *lfs, const lfd_
     for (int k = 0, b = 0; k < NSCLASS; k++) {
         ctx->cls_base[k] = b;
         b += ctx->cls_count[k];
+        int labels = 0, nnb = 0;
+        long long px = 0;
+        for (int v = 0; v < V; v++) {
+            if (hv[v].sclass != k) continue;
+            labels = std::max(labels, hv[v].L);
+            nnb = std::max(nnb, hv[v].nnb);
+            px += (long long)L.W[v] * L.H[v];
+        }
+        ctx->cls_bounded[k] = bounded_pays(k % 3, labels, nnb, px, ctx->cls_count[k], ctx->num_sms);
     }
     return LFD_OK;
 }
@@ -918,15 +955,13 @@ lfd_status rasterize_state(lfd_ctx *ctx, const float4 *planes, float *const *dep
 lfd_status run_sweep(lfd_ctx *ctx, float *cost, cudaStream_t st)
 {
     if (ctx->lc.sweep_persistent) LFD_CUDA(cudaMemsetAsync(ctx->d_queue, 0, 4 * QUEUE_INTS, st));
-    int bounded = ctx->lc.sweep_persistent;
-    for (const LfInfo &l : ctx->lfs) bounded = bounded && l.p.num_labels <= SWEEP_BOUNDED_LABELS;
     for (int k = 0; k < NSCLASS; k++) {
         if (!ctx->cls_count[k]) continue;
         const int threads = std::min(LCLASS_THREADS[k / 3], ctx->lc.sweep_threads);
         Consts c = ctx->c;                   // the class's pair form
         c.affine = k % 3 >= 1;
         c.shift = k % 3 == 2;
-        c.sweep_bounded = bounded;
+        c.sweep_bounded = ctx->lc.sweep_persistent && ctx->cls_bounded[k];
         LFD_CUDA(traced(ctx, LFD_STAGE_SWEEP, st, [&] {
             return launch_sweep(ctx->w, c, ctx->lc, threads, ctx->cls_base[k], ctx->cls_count[k], 4 + k,
                                 ctx->d_planesA, ctx->d_label, cost, st);
