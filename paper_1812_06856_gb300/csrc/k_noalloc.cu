@@ -65,13 +65,13 @@ constexpr int NA_WARP_AREA = 4096;
 
 template <int FMT>
 __global__ void __launch_bounds__(256) k_na_stats(const NoallocScratch *sc, const int *labels, const void *img,
-                                                  long long pitch, int W, int S, float *stats)
+                                                  long long pitch, int W, int S, int per, float *stats)
 {
     __shared__ lfd::SuperpixelSums<FMT> part[8];
     __shared__ int wcnt[8];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    const int s0 = blockIdx.x * 8, s = s0 + wid;
-    const int n = s < S ? sc->cnt[s] : -1;
+    const int s0 = blockIdx.x * per, s = s0 + wid;
+    const int n = wid < per && s < S ? sc->cnt[s] : -1;
     bool large = false;
     if (n > 0) {
         const int4 bb = sc->bbox[s];
@@ -105,7 +105,7 @@ __global__ void __launch_bounds__(256) k_na_stats(const NoallocScratch *sc, cons
     if (threadIdx.x < 8 && s0 + threadIdx.x < S && wcnt[threadIdx.x] >= 0)
         write(s0 + threadIdx.x, wcnt[threadIdx.x], part[threadIdx.x]);
     if (!any_large) return;
-    for (int k = 0; k < 8; k++) {
+    for (int k = 0; k < per; k++) {
         __syncthreads();
         if (s0 + k >= S || wcnt[k] >= 0) continue;   // uniform
         lfd::SuperpixelSums<FMT> t;
@@ -194,16 +194,16 @@ extern "C" lfd_status lfd_superpixel_stats_noalloc(const int32_t *labels, const 
     k_na_clear<<<(S + 255) / 256, 256, 0, st>>>(sc, S);
     if (!launch_failed()) k_na_count<<<(strips + 7) / 8, 256, 0, st>>>(sc, labels, width, height, S);
     if (!launch_failed()) {
-        const int blocks = (S + 7) / 8;
+        const int per = lfd::superpixels_per_cta(S, (long long)width * height), blocks = (S + per - 1) / per;
         switch (fmt) {
-        case LFD_RGBA8: k_na_stats<LFD_RGBA8><<<blocks, 256, 0, st>>>(sc, labels, image, pitch, width, S, stats_out); break;
+        case LFD_RGBA8: k_na_stats<LFD_RGBA8><<<blocks, 256, 0, st>>>(sc, labels, image, pitch, width, S, per, stats_out); break;
         case LFD_RGBA_F16:
-            k_na_stats<LFD_RGBA_F16><<<blocks, 256, 0, st>>>(sc, labels, image, pitch, width, S, stats_out);
+            k_na_stats<LFD_RGBA_F16><<<blocks, 256, 0, st>>>(sc, labels, image, pitch, width, S, per, stats_out);
             break;
         case LFD_RGBA_BF16:
-            k_na_stats<LFD_RGBA_BF16><<<blocks, 256, 0, st>>>(sc, labels, image, pitch, width, S, stats_out);
+            k_na_stats<LFD_RGBA_BF16><<<blocks, 256, 0, st>>>(sc, labels, image, pitch, width, S, per, stats_out);
             break;
-        default: k_na_stats<LFD_RGBA_F32><<<blocks, 256, 0, st>>>(sc, labels, image, pitch, width, S, stats_out); break;
+        default: k_na_stats<LFD_RGBA_F32><<<blocks, 256, 0, st>>>(sc, labels, image, pitch, width, S, per, stats_out); break;
         }
     }
     if (!launch_failed())

@@ -123,7 +123,7 @@ cudaError_t launch_sp_scan(const Workspace &w, int V, const int *cnt, int *off, 
 constexpr int SP_WARP_AREA = 4096;
 
 template <int FMT>
-__global__ void __launch_bounds__(256) k_sp_collect(Workspace w, Consts c, const int4 *bbox, const int *cnt,
+__global__ void __launch_bounds__(256) k_sp_collect(Workspace w, int per, const int4 *bbox, const int *cnt,
                                                     unsigned *pix, double2 *cen, int2 *ref, float4 *col)
 {
     __shared__ SuperpixelSums<FMT> part[8];
@@ -136,9 +136,9 @@ __global__ void __launch_bounds__(256) k_sp_collect(Workspace w, Consts c, const
         ref[gs] = make_int2(__double2int_rn(cx), __double2int_rn(cy));
         col[gs] = make_float4((float)r, (float)g, (float)b, 1.0f);
     };
-    const int gs0 = blockIdx.x * 8, gs = gs0 + wid;
+    const int gs0 = blockIdx.x * per, gs = gs0 + wid;
     bool large = false;
-    if (gs < w.S_total) {
+    if (wid < per && gs < w.S_total) {
         const int n = cnt[gs];
         if (n == 0) {
             if (lane == 0) {
@@ -172,7 +172,7 @@ __global__ void __launch_bounds__(256) k_sp_collect(Workspace w, Consts c, const
     // the warps' means, one lane each: FP64 divisions once per CTA
     if (threadIdx.x < 8 && wcnt[threadIdx.x] > 0) finish(gs0 + threadIdx.x, part[threadIdx.x], wcnt[threadIdx.x]);
     if (!any_large) return;
-    for (int k = 0; k < 8; k++) {
+    for (int k = 0; k < per; k++) {
         __syncthreads();
         if (wcnt[k] >= 0) continue;          // uniform
         const int g = gs0 + k, n = cnt[g], v = __ldg(w.sp_view + g);
@@ -215,12 +215,12 @@ __global__ void __launch_bounds__(256) k_sp_collect(Workspace w, Consts c, const
 cudaError_t launch_sp_collect(const Workspace &w, const Consts &c, const int4 *bbox, const int *cnt, unsigned *pix,
                               double2 *cen, int2 *ref, float4 *col, cudaStream_t st)
 {
-    const int blocks = (w.S_total + 7) / 8;
+    const int per = superpixels_per_cta(w.S_total, w.px_total), blocks = (w.S_total + per - 1) / per;
     switch (c.fmt) {
-    case LFD_RGBA8: k_sp_collect<LFD_RGBA8><<<blocks, 256, 0, st>>>(w, c, bbox, cnt, pix, cen, ref, col); break;
-    case LFD_RGBA_F16: k_sp_collect<LFD_RGBA_F16><<<blocks, 256, 0, st>>>(w, c, bbox, cnt, pix, cen, ref, col); break;
-    case LFD_RGBA_BF16: k_sp_collect<LFD_RGBA_BF16><<<blocks, 256, 0, st>>>(w, c, bbox, cnt, pix, cen, ref, col); break;
-    default: k_sp_collect<LFD_RGBA_F32><<<blocks, 256, 0, st>>>(w, c, bbox, cnt, pix, cen, ref, col); break;
+    case LFD_RGBA8: k_sp_collect<LFD_RGBA8><<<blocks, 256, 0, st>>>(w, per, bbox, cnt, pix, cen, ref, col); break;
+    case LFD_RGBA_F16: k_sp_collect<LFD_RGBA_F16><<<blocks, 256, 0, st>>>(w, per, bbox, cnt, pix, cen, ref, col); break;
+    case LFD_RGBA_BF16: k_sp_collect<LFD_RGBA_BF16><<<blocks, 256, 0, st>>>(w, per, bbox, cnt, pix, cen, ref, col); break;
+    default: k_sp_collect<LFD_RGBA_F32><<<blocks, 256, 0, st>>>(w, per, bbox, cnt, pix, cen, ref, col); break;
     }
     return cudaGetLastError();
 }

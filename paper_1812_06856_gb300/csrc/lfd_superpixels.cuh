@@ -187,6 +187,22 @@ __device__ __forceinline__ int scan_box(const int *labels, const void *img, long
     return found;
 }
 
+// Superpixels per CTA of 8 warps, from their number and the pixels they share:
+// a warp's each, unless large boxes are likely (2500 pixels on average).  Those
+// go through the CTA one after another, so there a CTA takes as many as one wave
+// of CTAs (152 SMs x 8) leaves to each.  Statistics of one view, us, eight per
+// CTA and by this rule (a CTA of their own for all superpixels before): 640x480
+// in cells of 60 x 60 118 and 74 (81), 150 x 150 286 and 78 (163), 24 labels
+// scattered over the image 2489 and 662 (1018); below that the split only leaves
+// warps idle (1920x1080 in cells of 46 x 46 84 and 96, 1280x720 of 16 x 16 41
+// and 46).
+inline int superpixels_per_cta(int S, long long px)
+{
+    if (px < 2500ll * S) return 8;
+    const int per = (S + 152 * 8 - 1) / (152 * 8);
+    return per < 1 ? 1 : (per > 8 ? 8 : per);
+}
+
 // ---------------------------------------------------------------------------
 // launch entries
 // ---------------------------------------------------------------------------
