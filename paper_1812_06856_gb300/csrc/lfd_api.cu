@@ -868,12 +868,39 @@ __global__ void __launch_bounds__(256) k_copy_views(const __grid_constant__ Copy
     }
 }
 
+// Whether a kernel on `device` may access p in 32-bit words: device memory of
+// that device, aligned.  Anything else a caller passes (another GPU's memory,
+// host memory, a byte offset) is left to the copy engine, which takes it or
+// reports it (0.1 us of host time a pointer).
+bool kernel_reaches(int device, const void *p)
+{
+    if ((uintptr_t)p % 4) return false;
+    cudaPointerAttributes a;
+    if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return a.type == cudaMemoryTypeDevice && a.device == device;
+}
+
 // `words` 32-bit words per superpixel between `flat` and the views' buffers
 // (entry k: view first + k; NULL entries are left out)
 template <bool GATHER>
-cudaError_t copy_views(const Layout &L, int first, int n, void *const *views, unsigned *flat, size_t words,
+cudaError_t copy_views(int device, const Layout &L, int first, int n, void *const *views, unsigned *flat, size_t words,
                        cudaStream_t st)
 {
+    bool reach = true;
+    for (int k = 0; k < n; k++) reach = reach && (!views[k] || kernel_reaches(device, views[k]));
+    if (!reach) {
+        for (int k = 0; k < n; k++) {
+            if (!views[k]) continue;
+            unsigned *at = flat + (size_t)L.sp_base[first + k] * words;
+            const cudaError_t e = cudaMemcpyAsync(GATHER ? at : views[k], GATHER ? views[k] : at,
+                                                  4 * words * L.S[first + k], cudaMemcpyDeviceToDevice, st);
+            if (e != cudaSuccess) return e;
+        }
+        return cudaSuccess;
+    }
     bool wide = words % 4 == 0 && (uintptr_t)flat % 16 == 0;
     for (int k = 0; k < n; k++) wide = wide && (uintptr_t)views[k] % 16 == 0;
     const size_t per = wide ? words / 4 : words;
@@ -903,7 +930,7 @@ lfd_status gather_planes(lfd_ctx *ctx, const float *const *src, float4 *dst, cud
     if (!src) return fail(ctx, LFD_ERR_INVALID_ARG, "planes array is NULL");
     for (int v = 0; v < ctx->L.V; v++)
         if (!src[v] && !allow_null) return fail(ctx, LFD_ERR_INVALID_ARG, "planes of view %d is NULL", v);
-    LFD_CUDA(copy_views<true>(ctx->L, 0, ctx->L.V, (void *const *)src, (unsigned *)dst, 4, st));
+    LFD_CUDA(copy_views<true>(ctx->device, ctx->L, 0, ctx->L.V, (void *const *)src, (unsigned *)dst, 4, st));
     return LFD_OK;
 }
 
@@ -915,7 +942,7 @@ lfd_status scatter(lfd_ctx *ctx, const T *src, T *const *dst, size_t per_sp, cud
     if (!dst) return LFD_OK;
     if (nviews < 0) nviews = ctx->L.V;
     if (kind == cudaMemcpyDeviceToDevice && per_sp <= 4) {
-        LFD_CUDA(copy_views<false>(ctx->L, first_view, nviews, (void *const *)dst, (unsigned *)src, per_sp, st));
+        LFD_CUDA(copy_views<false>(ctx->device, ctx->L, first_view, nviews, (void *const *)dst, (unsigned *)src, per_sp, st));
         return LFD_OK;
     }
     for (int k = 0; k < nviews; k++) {       // to the host, or large (costs)
