@@ -12,6 +12,7 @@
 
 #include "lfd_fuse.cuh"
 #include "lfd_internal.cuh"
+#include "lfd_kept.h"
 #include "lfd_slic.cuh"
 #include "lfd_superpixels.cuh"
 
@@ -233,9 +234,7 @@ struct lfd_ctx {
     std::vector<lfd_camera> cams;    // cameras of the bound views (global order)
     void *d_slic = nullptr;          // SLIC scratch (CIELAB image, centres)
     size_t slic_cap = 0;
-    unsigned *d_zbuf = nullptr;      // fusion z-buffers (one group of reference views at a time)
-    size_t zbuf_cap = 0;
-    bool zbuf_clean = false;         // every word is +inf once the enqueued work has run
+    KeptBuffer<unsigned> zbuf;       // fusion z-buffers (one group of reference views at a time), left at +inf
     void *d_ftab = nullptr;
     size_t ftab_cap = 0;
     // CUDA graph of a batched frame and the pinned depth table it reads
@@ -1351,7 +1350,7 @@ lfd_status lfd_destroy(lfd_ctx *ctx)
     ctx->stage.release();
     ctx->dtab.release();
     ctx->ftab.release();
-    if (ctx->d_zbuf) cudaFree(ctx->d_zbuf);
+    if (ctx->zbuf.p) cudaFree(ctx->zbuf.p);
     if (ctx->d_slic) cudaFree(ctx->d_slic);
     if (ctx->d_ftab) cudaFree(ctx->d_ftab);
     if (ctx->h_bdepth) cudaFreeHost(ctx->h_bdepth);
@@ -1739,16 +1738,16 @@ lfd_status lfd_fuse(lfd_ctx *ctx, const float *const *depth_in, float *const *de
         const size_t t = align_up(8 * (size_t)l.V, 16) + 8 * (size_t)l.V + 16 * (size_t)l.V + 48 * (size_t)l.V * l.V;
         tmax = std::max(tmax, t);
     }
-    const size_t zcap = ctx->zbuf_cap;
-    if ((s = ensure_dev(ctx, (void **)&ctx->d_zbuf, &ctx->zbuf_cap, align_up(4 * std::max<size_t>(zmax, 1), 16))) != LFD_OK)
-        return s;
+    s = ctx->zbuf.reserve(align_up(4 * std::max<size_t>(zmax, 1), 16),
+                          [&](void **p, size_t *cap, size_t bytes) { return ensure_dev(ctx, p, cap, bytes); });
+    if (s != LFD_OK) return s;
     if ((s = ensure_dev(ctx, &ctx->d_ftab, &ctx->ftab_cap, tmax)) != LFD_OK) return s;
     // under capture nothing runs yet: the graph clears for itself and the next call clears again
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     const bool capturing = cudaStreamIsCapturing(st, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone;
-    if (ctx->zbuf_cap != zcap || !ctx->zbuf_clean || capturing)
-        LFD_CUDA(traced(ctx, LFD_STAGE_FUSION, st, [&] { return launch_fuse_clear(ctx->d_zbuf, ctx->zbuf_cap, st); }));
-    ctx->zbuf_clean = false;                 // until every group that is started below is enqueued
+    if (!ctx->zbuf.clean || capturing)
+        LFD_CUDA(traced(ctx, LFD_STAGE_FUSION, st, [&] { return launch_fuse_clear(ctx->zbuf.p, ctx->zbuf.cap, st); }));
+    ctx->zbuf.clean = false;                 // until every group that is started below is enqueued
     for (size_t li = 0; li < ctx->lfs.size(); li++) {
         const LfInfo &l = ctx->lfs[li];
         const int V = l.V, f = l.first_view;
@@ -1818,12 +1817,12 @@ lfd_status lfd_fuse(lfd_ctx *ctx, const float *const *depth_in, float *const *de
         a.depth_in = (const float *const *)(d + o_in);
         a.depth_out = (float *const *)(d + o_out);
         a.mats = (const float *)(d + o_mats);
-        a.zbuf = ctx->d_zbuf;
+        a.zbuf = ctx->zbuf.p;
         for (const Group &g : groups[li])
             LFD_CUDA(traced(ctx, LFD_STAGE_FUSION, st,
                             [&] { return launch_fuse_group(a, g.first, g.count, max_w, max_h, max_px, st); }, 2));
     }
-    ctx->zbuf_clean = !capturing;
+    ctx->zbuf.clean = !capturing;
     return LFD_OK;
 }
 
