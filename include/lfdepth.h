@@ -264,7 +264,9 @@ lfd_status lfd_estimate_host(lfd_ctx *ctx, const lfd_lightfield *lf_host, const 
  *   device.  centres_in / centres_out (nullable; entries float[grid_w*grid_h*5]
  *   {L, a, b, x, y} on the device): start from given centres instead of the
  *   seeds / receive the centres the final assignment used.
- * Scratch is allocated in the context on first use.  Asynchronous. */
+ * Scratch is allocated in the context on first use, outside its budget: 16
+ * bytes per pixel (of the largest cell in every cell) and 472 per cell, for as
+ * many views at a time as fit 2 GB, at least one.  Asynchronous. */
 lfd_status lfd_slic(lfd_ctx *ctx, int32_t n, const void *const *views, const int64_t *view_pitch_bytes, int32_t fmt,
                     const int32_t *width, const int32_t *height, const int32_t *grid_w, const int32_t *grid_h,
                     double compactness, int32_t iterations, int32_t *const *labels_out,

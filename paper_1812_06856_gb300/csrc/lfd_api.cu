@@ -1858,18 +1858,28 @@ lfd_status lfd_slic(lfd_ctx *ctx, int32_t n, const void *const *views, const int
         if (pitch < (long long)width[v] * tb || pitch % tb)
             return fail(ctx, LFD_ERR_INVALID_ARG, "lfd_slic: view %d: bad pitch", v);
     }
-    // scratch for one group of up to SLIC_BATCH views at a time
-    size_t need = 0;
-    for (int g = 0; g < n; g += SLIC_BATCH) {
-        size_t sum = 0, o_c, sz_c;
-        for (int v = g; v < std::min(n, g + SLIC_BATCH); v++) sum += view_bytes(v, o_c, sz_c);
+    // scratch for one group of views at a time: up to SLIC_BATCH of them within SLIC_SCRATCH, at least one
+    auto group_end = [&](int g, size_t &sum) {
+        size_t o_c, sz_c;
+        int v = g;
+        for (sum = 0; v < std::min(n, g + SLIC_BATCH); v++) {
+            const size_t bytes = view_bytes(v, o_c, sz_c);
+            if (v > g && sum + bytes > SLIC_SCRATCH) break;
+            sum += bytes;
+        }
+        return v;
+    };
+    size_t need = 0, sum = 0;
+    for (int g = 0; g < n;) {
+        g = group_end(g, sum);
         need = std::max(need, sum);
     }
     if ((s = ensure_dev(ctx, &ctx->d_slic, &ctx->slic_cap, need)) != LFD_OK) return s;
     cudaStream_t st = (cudaStream_t)stream;
-    for (int g = 0; g < n; g += SLIC_BATCH) {
+    for (int g = 0, end = 0; g < n; g = end) {
         SlicBatch b = {};
-        b.n = std::min(n - g, SLIC_BATCH);
+        end = group_end(g, sum);
+        b.n = end - g;
         char *base = (char *)ctx->d_slic;
         for (int k = 0; k < b.n; k++) {
             const int v = g + k;

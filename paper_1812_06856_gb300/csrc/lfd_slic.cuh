@@ -20,6 +20,11 @@ struct SlicView {
 
 // up to SLIC_BATCH views segmented by the same launches (blockIdx.y = view)
 constexpr int SLIC_BATCH = 16;
+// Scratch of the views that go through the same launches.  A cell takes 432
+// bytes of sums, and 16 for each pixel of the largest cell: 41 bytes a pixel
+// for 5 x 5 cells, up to 540 for cells of one.  A group of this size is far
+// more work than the chip runs at once, so splitting there costs nothing.
+constexpr size_t SLIC_SCRATCH = (size_t)2 << 30;
 struct SlicBatch {
     SlicView v[SLIC_BATCH];
     float wxy[SLIC_BATCH];                // (m / S)^2 of each view
