@@ -222,6 +222,10 @@ lfd_status lfd_rasterize(lfd_ctx *ctx, const float *const *planes, float *const 
  *               (0 = current), refinement triangle (-1 = none) (nullable).
  *   energy_out: host array [V] of device float[2*S_v]: E after propagation and after
  *               refinement (nullable).
+ * Superpixels of 257 to 287 pixels: the sums of Eq. 9-11 run over 288 samples,
+ * the missing ones repeated at the rounded centroid (lfd_score sums the pixels
+ * alone); their energies differ from the definition by 0.06 % in the median, by
+ * 1 to 2 % in the worst hundredth.
  * Asynchronous. */
 lfd_status lfd_iterate(lfd_ctx *ctx, int32_t iter, const float *const *planes_in, float *const *planes_out,
                        int32_t *const *choice_out, float *const *energy_out, void *stream);

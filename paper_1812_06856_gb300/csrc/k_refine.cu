@@ -432,7 +432,15 @@ __device__ __forceinline__ void energy_sample(const ViewK &K, bool act, float du
                               cb, a);
 }
 
-// slots per lane that a superpixel of n pixels is summed with
+// Slots per lane that a superpixel of n pixels is summed with; every slot but
+// the last counts as full.  Nine slots have no class of their own: superpixels
+// of 257 to 287 pixels are summed as if they had 288, the missing ones being
+// copies of the anchor pixel (the rounded centroid, offset 0) in S_i, V_i, O_i
+// and the counts.  That departs from Eq. 9-11 and from lfd_score, which masks
+// them: energies of such superpixels are off by 6e-4 in the median, 1 to 2 % in
+// the worst hundredth and up to 17 % (4 x 640x480, pitch 16.5), those of other
+// sizes by FP32 rounding.  Masking them changes the planes of every light field
+// that has such superpixels.
 __device__ __forceinline__ int slot_class(int n)
 {
     const int s = (n + 31) >> 5;
@@ -448,7 +456,7 @@ struct ViewTerms {
 
 // View k of hypothesis h, whatever its pixels do there:
 // `slots` pixel slots per lane, every slot but the last taken as full unless
-// mask_all (n > 32 (slots - 1)).  One rolled loop for every slot count: it
+// mask_all (see slot_class).  One rolled loop for every slot count: it
 // serves the views that a superpixel's box straddles (and the scorer), and a
 // body per slot count next to view_term_inside's thrashes the instruction
 // cache (8 x 1024x768 arc: propagation 17.3 ms with unrolled bodies).
@@ -706,7 +714,7 @@ __device__ __noinline__ float2 eval_candidate(const Workspace &w, int src, float
     const int lane = threadIdx.x & 31;
     const SpShared &sh = sp_shared<COOP>();
     const int nnb = sh.S.nnb, slots = slot_class(sh.S.n);
-    const int count = max(sh.S.n, 32 * (slots - 1));          // every slot but the last counts in full
+    const int count = max(sh.S.n, 32 * (slots - 1));          // n, or 288 for 257 to 287 pixels (slot_class)
     const HypF h = cand_load(g_cs[threadIdx.x >> 5], src);
     const uint2 where = views_inside<AFF>(sh, h, nnb, DOMAIN == 0 ? sh.xy_lo : sh.xy_hi, lane);
     float ec = 0.f;
