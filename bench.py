@@ -44,6 +44,9 @@ import torch  # noqa: E402
 
 METRIC = "plane-hypothesis evals/s"
 UNIT = "evals/s"
+# what the value counts
+COUNTS = ("hypotheses decided: by their full sum, or by a bound that shows them to lose "
+          "(samples_taken_per_step of samples_per_step)")
 HEADLINE_CONFIG = 3
 L2_FLUSH_BYTES = 256 << 20
 # Algorithmic work per pixel-view sample of the two hot kernels.
@@ -422,7 +425,7 @@ def measure_frames(cfg: int, args, dev: str, local: int, ws: int, l2_peak: float
                            f"config{cfg}@{args.scale:g}", l2_peak)
     res = {"workload": workload_name(cfg, lf), "value": value, "ms_per_step": ms, "ms_per_view": ms / V,
            "samples_per_s": samples_per_s, "hypotheses_per_step": hyp_step, "samples_per_step": samples_step,
-           "samples_taken_per_step": sweep_samples + prop_samples,
+            "samples_taken_per_step": sweep_samples + prop_samples,
            "stage_ms": stage_ms, "wall_s": wall, "gpu_launches": int(sum(v[1] for v in prof.values())),
            "roofline": roofline, "clocks": clock_info}
 
@@ -523,11 +526,11 @@ def run_ours(args):
             "warmup": args.warmup, "ms_per_step": head["ms_per_step"], "higher_is_better": True,
             "scaling": "weak", "vs_baseline": None, "dtype": "f32", "data": "synthetic",
             "config": {"workload": head["workload"], "l2": "flushed between steps (256 MiB write)",
-                       "inputs": "device-resident", "parallelism": f"replicas x{ws}",
+                       "inputs": "device-resident", "parallelism": f"replicas x{ws}", "value_counts": COUNTS,
                        "storage": "FP16 views, FP32 accumulation" if cfg == 3 else "RGBA8 views, FP32 accumulation"},
             "ms_per_view": head["ms_per_view"]}
-    for k in ("samples_per_s", "hypotheses_per_step", "samples_per_step", "stage_ms", "wall_s", "gpu_launches",
-              "roofline", "clocks", "fusion", "slic", "e2e"):
+    for k in ("samples_per_s", "hypotheses_per_step", "samples_per_step", "samples_taken_per_step", "stage_ms", "wall_s",
+              "gpu_launches", "roofline", "clocks", "fusion", "slic", "e2e"):
         if k in head:
             line[k] = head[k]
     if rank == 0 and not args.no_cpu_baseline:
@@ -628,10 +631,10 @@ def run_ours_batch(args):
             "config": {"workload": mix_workload_name(len(mix), args.scale),
                        "superpixels": int(sum(m.rig.V * m.GW * m.GH for m in mix)),
                        "l2": "flushed between steps (256 MiB write)",
-                       "inputs": "device-resident", "parallelism": f"replicas x{ws}"},
+                       "inputs": "device-resident", "parallelism": f"replicas x{ws}", "value_counts": COUNTS},
             "samples_per_s": samples_per_s, "hypotheses_per_step": hyp_step,
             "samples_per_step": samples_step,
-           "samples_taken_per_step": sweep_samples + prop_samples, "stage_ms": stage_ms,
+            "samples_taken_per_step": sweep_samples + prop_samples, "stage_ms": stage_ms,
             "gpu_launches": int(sum(v[1] for v in prof.values())), "launch_config": ctx.launch_config(),
             "roofline": roofline, "clocks": clock_info, "input_generation_s": t_gen}
     # the same light fields through lfd_estimate one after another (the plain
