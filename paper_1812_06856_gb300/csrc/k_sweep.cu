@@ -13,8 +13,9 @@
 // the epipolar line; neighbouring labels therefore gather from neighbouring
 // texels (coalesced, L1-resident).  No reduction is needed per sample: each
 // thread owns its label's cost; a single block arg-min ends the CTA.  This
-// full sweep serves cost_out, world-frame sweeps, more than 256 labels and
-// the non-persistent launch shape; the others take the bounded sweep below.
+// full sweep serves cost_out, world-frame sweeps, more than 256 labels, the
+// non-persistent launch shape and sizes at which it is the faster one; the
+// others take the bounded sweep below.
 //
 // Homography per (label, view): for the plane g = z_k * gh (gh = (0,0,1) for
 // camera-frame sweeps) A = P + q g^T; its superpixel-anchored third column
@@ -356,7 +357,8 @@ __device__ __forceinline__ void sweep_sp(const Workspace &w, const Consts &c, in
 // pairs: its pipe is 16 times narrower than FP32's here.
 //
 // Measured against the full sweep (one thread per label): 16 x 1080p FP16,
-// 256 labels, 4 x 4 grid 104.6 -> 25.9 ms (24 % of the samples taken);
+// 256 labels, 4 x 4 grid 104.6 -> 25.9 ms (24 % of the samples taken; other
+// scenes of this size 21.9 to 27.5 ms with 20 to 25 %);
 // 8 x 1024x768 RGBA8, 256 labels, 30-degree arc 20.2 -> 13.5 ms (58 %: wide
 // baselines leave the best label a high cost, and the others go later).  What
 // bounds it: issue (64 % of the cycles) with the L1 data pipe at 66 % of its
@@ -936,9 +938,9 @@ static cudaError_t launch_sweep_f(const Workspace &w, const Consts &c, const Lau
                                   int count, int qidx, float4 *planes, int *label, float *cost, cudaStream_t st)
 {
     // arg-min only (no cost_out), camera frame, up to BS_LABELS labels (its
-    // shared-memory lists): the bounded sweep; measured above.  Costs need
-    // every label's full sum, world-frame sweeps and larger label counts keep
-    // the full sweep as well.
+    // shared-memory lists): the bounded sweep, where the class's sizes suit it
+    // (sweep_bounded).  Costs need every label's full sum, world-frame sweeps
+    // and larger label counts keep the full sweep as well.
     if (c.sweep_bounded && !cost && !c.sweep_frame) {
         if (c.affine && c.shift) return launch_bounded<FMT, PF_SHIFT>(w, lc, base, count, qidx, planes, label, st);
         if (c.affine) return launch_bounded<FMT, PF_AFFINE>(w, lc, base, count, qidx, planes, label, st);

@@ -92,7 +92,7 @@ struct Consts {
     int sweep_frame;
     int batch_iters;         // 1: a view whose light field has run its iterations passes its plane through
     float col_scale;         // sampler colour units -> [0,1]
-    int sweep_bounded;       // 1: a sweep without costs may drop labels that can no longer win (k_sweep_bounded)
+    int sweep_bounded;       // 1: a sweep without costs drops labels that can no longer win (k_sweep_bounded)
     int cand_batch;          // candidate planes per pass (16 or 32; LaunchCfg::prop_batch)
     int affine;              // 1: every pair's homography has third row (0, 0, c) for every plane
                              //    (parallel cameras, common principal depth axis): the sample's depth
